@@ -46,6 +46,16 @@ int grid_for(const void* kernel, int threads, size_t smem, int64_t work_items)
     return (int)(need < full ? need : full);
 }
 
+int line_stack_bytes(const void* kernel, int entries, size_t& bytes)
+{
+    bytes = (size_t)entries * sizeof(int);
+    // above 48 KB in total (trees of more than about 50 levels) a kernel needs leave
+    if (bytes > 24 * 1024)
+        WOB_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)bytes));
+    return WOB_OK;
+}
+
 int check_problem(const wob_problem* prob)
 {
     if (!prob || !prob->bvh) {
@@ -118,6 +128,7 @@ void fill_params(WalkParams& p, const wob_problem* prob, const float* queries,
     p.tv = b.tv;
     p.inv_order = b.inv_order;
     p.iter_limit = prob->iter_limit > 0 ? prob->iter_limit : (int)(4 * b.n_wide + 64);
+    p.stack_levels = b.wide_levels;
     p.verts = m.verts;
     p.verts_d = m.verts_d;
     p.tris = m.tris;
@@ -504,6 +515,7 @@ int wob_solve_forward(const wob_problem* prob, const float* queries, int64_t Q, 
     WOB_CUDA_TRY(cudaMallocAsync((void**)&sc.err, sizeof(Control), s));  // freed by sc
     WOB_CUDA_TRY(cudaMemsetAsync(sc.err, 0, sizeof(Control), s));
     p.error_word = &sc.err->err;
+    p.tile_counter = &sc.err->next_tile;
     double* zp = zpos;
     double* w = zw;
     double* own = nullptr;

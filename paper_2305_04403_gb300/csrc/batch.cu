@@ -25,14 +25,14 @@
 #include <sys/stat.h>
 #include <unistd.h>
 
-#include "wob_device.cuh"
+#include "line_engine.cuh"
 #include "wob_host.h"
 
 namespace wob {
 
 namespace {
 
-constexpr unsigned kFull = 0xFFFFFFFFu;
+constexpr unsigned kFull = kAllLanes;
 
 struct BatchProblem {
     const float4* nodes;  // 8-wide nodes
@@ -57,50 +57,102 @@ struct Tile {
     int64_t first;  // first walk (problem-local)
 };
 
+// The engine's policy for a batch: a fetched tile (32 x ROUNDS consecutive
+// walks of one problem) is handed to the engine 32 walks at a time; the two
+// slots may belong to different problems.
 template <int ROUNDS>
-__global__ void __launch_bounds__(128, 8)
-    k_dl_batched(const BatchProblem* __restrict__ probs, const Tile* __restrict__ tiles,
+struct BatchWalks {
+    const BatchProblem* probs;
+    const Tile* tiles;
+    int64_t n_tiles;
+    const float* queries;
+    unsigned long long* counter;
+    double* part;
+    uint64_t seed;
+    Tile t0{0, 0, 0}, t1{0, 0, 0};  // the problem and first walk of either slot
+    int left = 0;                   // rounds left of the newest tile
+    int newest = 0;
+    __device__ __forceinline__ bool fetch(int slot, int& cnt)
+    {
+        Tile t;
+        if (left > 0) {
+            t = newest ? t1 : t0;
+            t.first += 32;
+            --left;
+        } else {
+            unsigned long long i = 0;
+            if ((threadIdx.x & 31) == 0) i = atomicAdd(counter, 1ull);
+            i = __shfl_sync(kFull, i, 0);
+            if (i >= (unsigned long long)n_tiles) return false;
+            t = tiles[i];
+            left = ROUNDS - 1;
+        }
+        const int64_t rest = probs[t.problem].n_walks - t.first;
+        cnt = rest >= 32 ? 32 : (rest > 0 ? (int)rest : 0);
+        if (rest <= 32) left = 0;
+        newest = slot;
+        if (slot) t1 = t; else t0 = t;
+        return true;
+    }
+    __device__ __forceinline__ const BatchProblem& prob(const LaneWalk& lw) const
+    {
+        return probs[lw.id < 32 ? t0.problem : t1.problem];
+    }
+    __device__ __forceinline__ StreamKey key(const LaneWalk& lw) const
+    {
+        return {(uint32_t)seed ^ prob(lw).problem, (uint32_t)(seed >> 32)};
+    }
+    __device__ __forceinline__ LineGeom geom(const LaneWalk& lw) const
+    {
+        const BatchProblem& P = prob(lw);
+        return {P.nodes, P.tv, P.edge_thr_L, P.tauL, P.graze, P.iter_limit};
+    }
+    __device__ __forceinline__ void begin(const LaneMem& mem, LaneWalk& lw)
+    {
+        const BatchProblem& P = prob(lw);
+        const int64_t local = (lw.id < 32 ? t0.first : t1.first) + (lw.id & 31);
+        const int64_t qi = local / P.N;
+        mem.set_ids((uint32_t)qi, (uint32_t)(local - qi * P.N));
+        const float* qp = queries + 3 * (P.query_base + qi);
+        dl_begin(mem, lw, make_float3(qp[0], qp[1], qp[2]), -1, P.data, P.tv, (double)P.phi, P.M);
+    }
+    __device__ __forceinline__ bool depart(const LaneMem&, const LaneWalk&) const { return true; }
+    __device__ __forceinline__ bool land(const LaneMem& mem, LaneWalk& lw, int m, int pos, int)
+    {
+        if (m == 0) return false;
+        const BatchProblem& P = prob(lw);
+        dl_land(mem, lw, m, pos, P.data, P.tv, (double)P.phi, P.M);
+        return lw.k < P.M;
+    }
+    __device__ __forceinline__ double value(const LaneMem& mem, const LaneWalk&) const
+    {
+        return mem.get(kAccS);
+    }
+    __device__ __forceinline__ void close(int slot, int cnt, double v) const
+    {
+        const Tile& t = slot ? t1 : t0;
+        const BatchProblem& P = probs[t.problem];
+        const int lane = threadIdx.x & 31;
+        const bool live = lane < cnt;
+        const int64_t local = t.first + lane;
+        const int64_t qi = live ? local / P.N : 0;
+        add_tile_partials(v, live, qi, local - qi * P.N, (P.N + 31) / 32, part + 2 * P.part_base);
+    }
+};
+
+template <int ROUNDS>
+__global__ void __launch_bounds__(kLineThreads, 6)
+    k_batch_lines(const BatchProblem* __restrict__ probs, const Tile* __restrict__ tiles,
                  int64_t n_tiles, const float* __restrict__ queries,
                  const uint64_t* __restrict__ seed_dev, unsigned long long* counter,
-                 double* __restrict__ part, int* err_word)
+                 double* __restrict__ part, int* err_word, int levels)
 {
-    const int lane = threadIdx.x & 31;
-    const uint64_t seed = *seed_dev;
-    __shared__ double slots[8 * 128];
-    __shared__ int leafq[kLeafQ * 128];
-    const WalkSlot ws{slots + threadIdx.x, 128};
-    const LeafQueue lq{leafq + threadIdx.x, 128};
-    int stack[kStackSize];
-    int hits[kMaxHits];
+    __shared__ LineShared sm;
+    extern __shared__ int line_stack[];
     int err = 0;
     WalkCount c{0, 0, 0, 0, 0};
-    while (true) {
-        unsigned long long t = 0;
-        if (lane == 0) t = atomicAdd(counter, 1ull);
-        t = __shfl_sync(kFull, t, 0);
-        if (t >= (unsigned long long)n_tiles) break;
-        const Tile tile = tiles[t];
-        const BatchProblem& P = probs[tile.problem];
-        const DLGeom G{P.nodes, P.tv, P.iter_limit, P.edge_thr_L, P.tauL, P.graze};
-        const StreamKey key{(uint32_t)seed ^ P.problem, (uint32_t)(seed >> 32)};
-#pragma unroll 1
-        for (int r = 0; r < ROUNDS; ++r) {
-            const int64_t local = tile.first + r * 32 + lane;
-            const bool live = local < P.n_walks;
-            const int64_t qi = live ? local / P.N : 0;
-            const int64_t w = local - qi * P.N;
-            double v = 0.0;
-            if (live) {
-                const float* qp = queries + 3 * (P.query_base + qi);
-                const double3 x = make_double3(qp[0], qp[1], qp[2]);
-                int wflag = 0;
-                v = dl_walk<false, false>(G, P.data, (double)P.phi, P.M, key, (uint32_t)qi,
-                                          (uint32_t)w, x, -1, ws, stack, hits, err, wflag,
-                                          LineOut{nullptr, nullptr, nullptr}, c, lq);
-            }
-            add_tile_partials(v, live, qi, w, (P.N + 31) / 32, part + 2 * P.part_base);
-        }
-    }
+    BatchWalks<ROUNDS> pol{probs, tiles, n_tiles, queries, counter, part, *seed_dev};
+    run_lines<BatchWalks<ROUNDS>, false>(pol, sm.lane(line_stack), sm.vals, levels, err, c);
     if (err) atomicOr(err_word, err);
 }
 
@@ -216,6 +268,7 @@ struct wob_batch_s {
     int32_t P = 0;
     int64_t Qt = 0, W = 0, max_lines = 0;
     int64_t n_slots = 0;  // (query, 32-walk block) slots of all problems
+    int levels = 1;       // levels of the deepest problem's tree
     std::vector<BatchProblem> host_probs;
     std::vector<int32_t> walks;
     std::vector<int64_t> qoff, part_base;
@@ -257,28 +310,35 @@ std::vector<Tile> make_tiles(const wob_batch_s& b, const std::vector<double>& co
     return t;
 }
 
-int batch_grid(int rounds, int64_t n_tiles)
+const void* batch_kernel(int rounds)
 {
-    const void* kern = rounds == 4 ? (const void*)k_dl_batched<4>
-                     : rounds == 2 ? (const void*)k_dl_batched<2> : (const void*)k_dl_batched<1>;
-    return grid_for(kern, 128, 0, n_tiles * 32);
+    return rounds == 4 ? (const void*)k_batch_lines<4>
+           : rounds == 2 ? (const void*)k_batch_lines<2> : (const void*)k_batch_lines<1>;
+}
+
+// Grid and dynamic shared memory of a launch (sets the kernel's limit:
+// before any capture).
+int batch_grid(const wob_batch_s& b, int rounds, int64_t n_tiles, int& grid, size_t& smem)
+{
+    WOB_TRY(line_stack_bytes(batch_kernel(rounds), b.levels * kLineThreads, smem));
+    grid = grid_for(batch_kernel(rounds), kLineThreads, smem, n_tiles * 32);
+    return WOB_OK;
 }
 
 // Counter reset + walk kernel (no API call here may break stream capture).
 int launch_batch_kernels(wob_batch_s& b, const BatchProblem* probs, const Tile* tiles,
-                         int64_t n_tiles, int rounds, int grid, double* part, int64_t n_slots,
-                         cudaStream_t s)
+                         int64_t n_tiles, int rounds, int grid, size_t smem, double* part,
+                         int64_t n_slots, cudaStream_t s)
 {
     WOB_CUDA_TRY(cudaMemsetAsync(b.counter, 0, sizeof(unsigned long long), s));
     WOB_CUDA_TRY(cudaMemsetAsync(b.err, 0, sizeof(int), s));  // this run's checks
     WOB_CUDA_TRY(cudaMemsetAsync(part, 0, n_slots * 2 * sizeof(double), s));  // added into
-    const int threads = 128;
     if (rounds == 4)
-        k_dl_batched<4><<<grid, threads, 0, s>>>(probs, tiles, n_tiles, b.queries, b.seed_dev, b.counter, part, b.err);
+        k_batch_lines<4><<<grid, kLineThreads, smem, s>>>(probs, tiles, n_tiles, b.queries, b.seed_dev, b.counter, part, b.err, b.levels);
     else if (rounds == 2)
-        k_dl_batched<2><<<grid, threads, 0, s>>>(probs, tiles, n_tiles, b.queries, b.seed_dev, b.counter, part, b.err);
+        k_batch_lines<2><<<grid, kLineThreads, smem, s>>>(probs, tiles, n_tiles, b.queries, b.seed_dev, b.counter, part, b.err, b.levels);
     else
-        k_dl_batched<1><<<grid, threads, 0, s>>>(probs, tiles, n_tiles, b.queries, b.seed_dev, b.counter, part, b.err);
+        k_batch_lines<1><<<grid, kLineThreads, smem, s>>>(probs, tiles, n_tiles, b.queries, b.seed_dev, b.counter, part, b.err, b.levels);
     WOB_CUDA_TRY(cudaGetLastError());
     return WOB_OK;
 }
@@ -328,11 +388,13 @@ int autotune(wob_batch_s& b, const std::vector<double>& cost, cudaStream_t s)
             }
             cudaMemcpy(dt, t.data(), t.size() * sizeof(Tile), cudaMemcpyHostToDevice);
             float ms = 0.f, best_rep = 1e30f;
+            int grid = 1;
+            size_t smem = 0;
+            rc = batch_grid(b, rounds_c[ri], (int64_t)t.size(), grid, smem);
             for (int rep = 0; rep < 2 && rc == WOB_OK; ++rep) {  // first run warms caches
                 cudaEventRecord(e0, s);
-                rc = launch_batch_kernels(b, dprobs, dt, (int64_t)t.size(), rounds_c[ri],
-                                          batch_grid(rounds_c[ri], (int64_t)t.size()), b.part,
-                                          base, s);
+                rc = launch_batch_kernels(b, dprobs, dt, (int64_t)t.size(), rounds_c[ri], grid,
+                                          smem, b.part, base, s);
                 cudaEventRecord(e1, s);
                 cudaEventSynchronize(e1);
                 cudaEventElapsedTime(&ms, e0, e1);
@@ -407,6 +469,7 @@ int wob_batch_create(const wob_problem* problems, int32_t P, const int64_t* quer
         bp.tv = wp.tv;
         bp.data = wp.data;
         bp.iter_limit = wp.iter_limit;
+        b->levels = std::max(b->levels, wp.stack_levels);
         bp.phi = wp.phi;
         bp.M = max_len[p];
         bp.N = walks[p];
@@ -503,11 +566,13 @@ int wob_batch_create(const wob_problem* problems, int32_t P, const int64_t* quer
         set_error("wob_batch_create: stream creation failed");
         return fail(WOB_ERR_CUDA);
     }
-    const int g_walk = batch_grid(b->rounds, b->n_tiles);
+    int g_walk = 1;
+    size_t smem = 0;
+    if ((rc = batch_grid(*b, b->rounds, b->n_tiles, g_walk, smem)) != WOB_OK) return fail(rc);
     const int g_red = grid_for((const void*)k_reduce_batched, 256, 0, b->Qt * 32);
     cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal);
-    rc = launch_batch_kernels(*b, b->probs, b->tiles, b->n_tiles, b->rounds, g_walk, b->part,
-                              b->n_slots, b->cap_stream);
+    rc = launch_batch_kernels(*b, b->probs, b->tiles, b->n_tiles, b->rounds, g_walk, smem,
+                              b->part, b->n_slots, b->cap_stream);
     if (rc == WOB_OK && b->Qt > 0)
         k_reduce_batched<<<g_red, 256, 0, b->cap_stream>>>(b->part, b->qoff_dev,
                                                            b->part_base_dev, b->walks_dev, P,

@@ -1,27 +1,28 @@
 // walk.cu -- the walk-on-boundary kernels:
-//   k_dl_walks   Dirichlet problems, double-layer formulation, ray (line)
+//   k_dl_lines   Dirichlet problems, double-layer formulation, ray (line)
 //                sampling with all-hits queries (Sec. 4.1, 4.4.1)
 //   k_sl_walks_ff / k_sl_walks
 //                Neumann / Robin problems, single-layer formulation, area
 //                sampling / resampled importance sampling (Sec. 4.3)
-//   k_nd_walks   Neumann problems through the direct boundary integral
+//   k_nd_lines   Neumann problems through the direct boundary integral
 //                equation (Sec. 4.2)
 //   k_reduce*    per-query FP64 mean and variance (Sec. 4.1.1)
 // plus the debug kernels behind wob_trace_lines / wob_line_axes /
 // wob_philox4x32_10.
 //
-// One thread owns one walk from start to end; the walk values of a warp's 32
-// walks are summed per query in a fixed order into (sum, sum of squares)
-// partials (add_tile_partials), which k_reduce_part combines per query in a
-// fixed order, so results do not depend on scheduling.  Debug solves also
-// write every walk's value.
+// One thread owns one walk (line walks of calls with few walks: a group of
+// lanes, line_engine.cuh); the values of 32 consecutive walks are summed per
+// query in a fixed order into (sum, sum of squares) partials
+// (add_tile_partials), which k_reduce_part combines per query in a fixed
+// order, so results do not depend on scheduling.  Debug solves also write
+// every walk's value.
 #include <cmath>
 #include <cstddef>
 #include <cstdlib>
 
 #include "bits.cuh"
 #include "ff.cuh"
-#include "wob_device.cuh"
+#include "line_engine.cuh"
 #include "wob_host.h"
 
 namespace wob {
@@ -30,9 +31,20 @@ namespace {
 
 constexpr double kFourPi = 12.566370614359172953850573533118;
 
-#ifndef WOB_DL_MIN_BLOCKS
-#define WOB_DL_MIN_BLOCKS 8
-#endif
+// Line walks: six blocks of 128 threads per SM (80 registers; see
+// line_engine.cuh), 24 warps of the grouped form; the forms that need more
+// registers than that to keep out of local memory get fewer blocks.
+constexpr int kLineBlocks = 6;
+constexpr int kNdBlocks = 7;  // direct BIE: 72 registers hold it (22.7 -> 21.4 ms on the torus)
+constexpr int kDebugBlocks = 4;
+constexpr int kGroupBlocks = 24 / kG;
+// Calls of at most this many walks per SM run with a group of lanes per walk.
+// 32,768 walks (216 per SM) took the group and the single lane 150 and 158 us
+// (4 lines each, 1,280 triangles), 1,318 and 1,262 us (16 lines, 81,920) and
+// 1,035 and 997 us (direct BIE, 12 lines); half as many 98 against 153, 772
+// against 1,160 and 633 against 938 us; twice as many 226 against 205, 2,064
+// against 1,454 and 1,608 against 1,153 us.
+constexpr int64_t kGroupWalksPerSm = 200;
 // Single-layer walks with area sampling: 6 blocks of 128 threads per SM (71
 // registers, no spills) hide the latency of the CDF search better than the
 // unbounded 121 registers (4 blocks; 8% slower) or 8 blocks (64 registers,
@@ -41,71 +53,174 @@ constexpr double kFourPi = 12.566370614359172953850573533118;
 #define WOB_SL_MIN_BLOCKS 6
 #endif
 
-// One thread owns one walk; warps take tiles of 32 consecutive walks from a
-// global counter until none are left (dynamic balance; consecutive walks of
-// a query start their first lines at the same point).  Per line:
-// draw the axis, traverse (descend to a leaf, test it, repeat), then pick
-// the hit (keys only when m > 1), refine it in float-float and add the
-// data term (evaluated in FP32) to the FP64 walk sum.  The kernel is
-// limited to 64 registers (8 blocks of 128 threads per SM): the traversal
-// is latency-bound and occupancy pays more than the few values the
-// compiler keeps in local memory.  Lanes that start their lines
-// together share the fetches of the upper tree levels; variants that broke
-// this (persistent lanes refilled from a global counter, or a wavefront of
-// separate traversal and FP64-update kernels) measured 8-18% slower.
-template <bool COUNT, bool DEBUG, bool GRAD = false>
-__global__ void __launch_bounds__(128, WOB_DL_MIN_BLOCKS) k_dl_walks(WalkParams p)
-{
-    const StreamKey key{p.key0, p.key1};
-    const int64_t total = p.Q * (int64_t)p.N;
-    const DLGeom G{p.nodes, p.tv, p.iter_limit, p.edge_thr_L, p.tauL, p.graze};
-    __shared__ double slots[(GRAD ? 11 : 8) * 128];
-    __shared__ int leafq[kLeafQ * 128];
-    const WalkSlot ws{slots + threadIdx.x, 128};
-    const LeafQueue lq{leafq + threadIdx.x, 128};
-    int err = 0;
-    int stack[kStackSize];
-    int hits[kMaxHits];
-    WalkCount c{0, 0, 0, 0, 0};
-    const int lane = threadIdx.x & 31;
-    while (true) {
-        // a warp takes the next 32 consecutive walks (one atomic per warp)
-        unsigned long long tile = 0;
-        if (lane == 0) tile = atomicAdd(p.tile_counter, 1ull);
-        tile = __shfl_sync(0xFFFFFFFFu, tile, 0);
-        if ((int64_t)tile * 32 >= total) break;
-        const int64_t idx = (int64_t)tile * 32 + lane;
-        const bool live = idx < total;
-        const int64_t qi = live ? idx / p.N : 0;
-        const int64_t wi = idx - qi * p.N;
-        double v = 0.0;
-        if (live) {
-            const uint32_t q = p.q_base + (uint32_t)qi;
-            const uint32_t w = (uint32_t)(p.walk_begin + wi);
-            const double3 x =
-                make_double3(p.queries[3 * qi], p.queries[3 * qi + 1], p.queries[3 * qi + 2]);
-            int wflag = 0;
-            int start = -1;
-            if (p.query_prim) {  // density walks from boundary points
-                const int32_t prim = p.query_prim[qi];
-                start = (prim >= 0 && prim < p.T) ? p.inv_order[prim] : -1;
-            }
-            const int64_t lk = idx * p.M;
-            const LineOut lo{DEBUG && p.line_m ? p.line_m + lk : nullptr,
-                             DEBUG && p.line_prim ? p.line_prim + lk : nullptr,
-                             DEBUG && p.line_flag ? p.line_flag + lk : nullptr};
-            v = dl_walk<COUNT, DEBUG, GRAD, GRAD>(G, p.data, (double)p.phi, p.M, key, q, w, x,
-                                                  start, ws, stack, hits, err, wflag, lo, c, lq);
-            if (p.per_walk) p.per_walk[idx] = v;
-            if (GRAD) {  // gradient of the same walk: first-step factor x walk value
-                p.per_walk_grad[idx] = ws.get(8) * v;
-                p.per_walk_grad[total + idx] = ws.get(9) * v;
-                p.per_walk_grad[2 * total + idx] = ws.get(10) * v;
-            }
-            if (DEBUG && p.walk_flag) p.walk_flag[idx] = (uint8_t)wflag;
-        }
-        if (p.part) add_tile_partials(v, live, qi, wi, p.tpq, p.part);
+// Tiles of 32 consecutive walks of one problem from its global counter
+// (dynamic balance), the 64-bit bookkeeping of the two tiles under way and
+// the per-tile sums: what the engine's single-problem policies share.
+struct WalkTiles {
+    const WalkParams& p;
+    int64_t total;
+    int64_t first0 = 0, first1 = 0;  // first walk of the tile in either slot
+    __device__ __forceinline__ explicit WalkTiles(const WalkParams& p_)
+        : p(p_), total(p_.Q * (int64_t)p_.N)
+    {
     }
+    __device__ __forceinline__ bool take(unsigned long long tile, int slot, int& cnt)
+    {
+        const int64_t first = (int64_t)tile * 32;
+        if (first >= total) return false;
+        if (slot) first1 = first; else first0 = first;
+        cnt = total - first < 32 ? (int)(total - first) : 32;
+        return true;
+    }
+    __device__ __forceinline__ bool fetch(int slot, int& cnt)
+    {
+        unsigned long long tile = 0;
+        if ((threadIdx.x & 31) == 0) tile = atomicAdd(p.tile_counter, 1ull);
+        return take(__shfl_sync(kAllLanes, tile, 0), slot, cnt);
+    }
+    // a tile for the whole block (into slot 0)
+    __device__ __forceinline__ bool fetch_block(unsigned long long* shared, int& cnt)
+    {
+        if (threadIdx.x == 0) *shared = atomicAdd(p.tile_counter, 1ull);
+        __syncthreads();
+        const unsigned long long tile = *shared;
+        __syncthreads();
+        return take(tile, 0, cnt);
+    }
+    __device__ __forceinline__ int64_t index(const LaneWalk& lw) const
+    {
+        return (lw.id < 32 ? first0 : first1) + (lw.id & 31);
+    }
+    // stream ids and coordinates of the walk's query; returns the query's row
+    template <class Mem>
+    __device__ __forceinline__ int64_t start(const Mem& mem, const LaneWalk& lw, float3& x) const
+    {
+        const int64_t idx = index(lw);
+        const int64_t qi = idx / p.N;
+        mem.set_ids(p.q_base + (uint32_t)qi, (uint32_t)(p.walk_begin + (idx - qi * p.N)));
+        x = make_float3(p.queries[3 * qi], p.queries[3 * qi + 1], p.queries[3 * qi + 2]);
+        return qi;
+    }
+    __device__ __forceinline__ void close(int slot, int cnt, double v) const
+    {
+        if (!p.part) return;
+        const int lane = threadIdx.x & 31;
+        const bool live = lane < cnt;
+        const int64_t idx = (slot ? first1 : first0) + lane;
+        const int64_t qi = live ? idx / p.N : 0;
+        add_tile_partials(v, live, qi, idx - qi * p.N, p.tpq, p.part);
+    }
+    __device__ __forceinline__ StreamKey key(const LaneWalk&) const { return {p.key0, p.key1}; }
+    __device__ __forceinline__ LineGeom geom(const LaneWalk&) const
+    {
+        return {p.nodes, p.tv, p.edge_thr_L, p.tauL, p.graze, p.iter_limit};
+    }
+    // debug solves: per-line outputs of the walk
+    __device__ __forceinline__ LineOut lines(const LaneWalk& lw) const
+    {
+        const int64_t lk = index(lw) * p.M;
+        return {p.line_m ? p.line_m + lk : nullptr, p.line_prim ? p.line_prim + lk : nullptr,
+                p.line_flag ? p.line_flag + lk : nullptr};
+    }
+};
+
+// Dirichlet walks (double layer) of one problem.
+template <bool DEBUG, bool GRAD>
+struct DlWalks : WalkTiles {
+    using Base = WalkTiles;
+    using Base::p;
+    __device__ __forceinline__ explicit DlWalks(const WalkParams& p_) : Base(p_) {}
+    template <class Mem>
+    __device__ __forceinline__ void begin(const Mem& mem, LaneWalk& lw)
+    {
+        float3 x;
+        const int64_t qi = Base::start(mem, lw, x);
+        int start = -1;
+        if (p.query_prim) {  // density walks from boundary points
+            const int32_t prim = p.query_prim[qi];
+            start = (prim >= 0 && prim < p.T) ? p.inv_order[prim] : -1;
+        }
+        dl_begin(mem, lw, x, start, p.data, p.tv, (double)p.phi, p.M);
+        if (GRAD) p.per_walk[Base::index(lw)] = __hiloint2double(0, -1);  // no first hit yet
+        if (DEBUG) {
+            const LineOut lo = Base::lines(lw);
+            for (int k = 0; k < p.M; ++k) lo.put(k, -1, -1, 0);
+        }
+    }
+    template <class Mem>
+    __device__ __forceinline__ bool depart(const Mem&, const LaneWalk& lw) const
+    {
+        return lw.k < p.M;
+    }
+    template <class Mem>
+    __device__ __forceinline__ bool land(const Mem& mem, LaneWalk& lw, int m, int pos, int flag)
+    {
+        if (DEBUG) {
+            lw.flag |= flag;
+            Base::lines(lw).put(lw.k, m, pos >= 0 ? (int)prim_of(p.tv, pos) : -1, flag);
+        }
+        if (m == 0) return false;
+        const bool first = GRAD && lw.k == 0;
+        dl_land(mem, lw, m, pos, p.data, p.tv, (double)p.phi, p.M);
+        if (first) park(Base::index(lw), pos, mem.x(0), mem.x(1), mem.x(2));
+        return lw.k < p.M;
+    }
+    template <class Mem>
+    __device__ __forceinline__ double value(const Mem& mem, const LaneWalk& lw) const
+    {
+        const double v = mem.get(kAccS);
+        if (DEBUG) {
+            const int64_t idx = Base::index(lw);
+            if (p.per_walk) p.per_walk[idx] = v;
+            if (p.walk_flag) p.walk_flag[idx] = (uint8_t)lw.flag;
+        }
+        return v;
+    }
+    // The first hit of a walk waits in the walk's own output slots until its
+    // tile is complete: its gradient factor takes FP64 square roots and
+    // divisions, which cost the warp the same for one lane as for 32.
+    __device__ __forceinline__ void park(int64_t idx, int pos, ff y0, ff y1, ff y2) const
+    {
+        const ff y[3] = {y0, y1, y2};
+        p.per_walk[idx] = __hiloint2double(0, pos);
+        for (int c = 0; c < 3; ++c)
+            p.per_walk_grad[c * Base::total + idx] =
+                __hiloint2double(__float_as_int(y[c].hi), __float_as_int(y[c].lo));
+    }
+    __device__ __forceinline__ void close(int slot, int cnt, double v) const
+    {
+        Base::close(slot, cnt, v);
+        const int lane = threadIdx.x & 31;
+        if (GRAD && lane < cnt) {  // gradient of a walk: first-step factor x walk value
+            const int64_t idx = (slot ? Base::first1 : Base::first0) + lane;
+            const int pos = __double2loint(p.per_walk[idx]);
+            double3 g = make_double3(0.0, 0.0, 0.0);
+            if (pos >= 0) {
+                double y[3];
+                for (int c = 0; c < 3; ++c) {
+                    const double b = p.per_walk_grad[c * Base::total + idx];
+                    y[c] = ff_join({__int_as_float(__double2hiint(b)), __int_as_float(__double2loint(b))});
+                }
+                const float* x = p.queries + 3 * (idx / p.N);
+                g = grad_factor(p.tv, pos, make_double3(x[0], x[1], x[2]), make_double3(y[0], y[1], y[2]));
+            }
+            p.per_walk[idx] = v;
+            p.per_walk_grad[idx] = g.x * v;
+            p.per_walk_grad[Base::total + idx] = g.y * v;
+            p.per_walk_grad[2 * Base::total + idx] = g.z * v;
+        }
+    }
+};
+
+template <bool COUNT, bool DEBUG, bool GRAD>
+__global__ void __launch_bounds__(kLineThreads, DEBUG ? kDebugBlocks : kLineBlocks) k_dl_lines(WalkParams p)
+{
+    __shared__ LineShared sm;
+    extern __shared__ int line_stack[];
+    int err = 0;
+    WalkCount c{0, 0, 0, 0, 0};
+    DlWalks<DEBUG, GRAD> pol(p);
+    run_lines<DlWalks<DEBUG, GRAD>, COUNT>(pol, sm.lane(line_stack), sm.vals, p.stack_levels, err, c);
     if (err) atomicOr(p.error_word, err);
     if (COUNT) {
         atomicAdd(p.counters + 0, c.lines);
@@ -114,6 +229,17 @@ __global__ void __launch_bounds__(128, WOB_DL_MIN_BLOCKS) k_dl_walks(WalkParams 
         atomicAdd(p.counters + 3, c.hits);
         atomicAdd(p.counters + 4, c.flag);
     }
+}
+
+template <bool GRAD>
+__global__ void __launch_bounds__(kGroupThreads, kGroupBlocks) k_dl_groups(WalkParams p)
+{
+    __shared__ GroupShared sm;
+    extern __shared__ int line_stack[];
+    int err = 0;
+    DlWalks<false, GRAD> pol(p);
+    run_line_groups(pol, sm, line_stack, p.stack_levels, err);
+    if (err) atomicOr(p.error_word, err);
 }
 
 // Data of the single-layer problems at y on triangle j (original order):
@@ -575,118 +701,112 @@ __global__ void __launch_bounds__(128, WOB_SL_MIN_BLOCKS) k_sl_walks_ff(WalkPara
 // boundary vertex, as the double-layer walks).  A query on triangle
 // query_prim is boundary vertex 1 with weight 1.  One thread per walk.
 template <bool DEBUG>
-__global__ void __launch_bounds__(128, WOB_DL_MIN_BLOCKS) k_nd_walks(WalkParams p)
-{
-    const StreamKey key{p.key0, p.key1};
-    const int64_t total = p.Q * (int64_t)p.N;
-    const double phi = (double)p.phi;
-    const float phi_f = (float)p.phi, area_f = (float)p.area;
-    const float rmin2 = (float)(1e-24 * p.L * p.L);
-    // walk state (point and axis as float-float pairs, S and P in FP64)
-    // parked in shared memory during the traversal (as in k_dl_walks), which
-    // leaves the postponed-leaf traversal its registers
-    __shared__ double slots[8 * 128];
-    __shared__ int leafq[kLeafQ * 128];
-    const WalkSlot ws{slots + threadIdx.x, 128};
-    const LeafQueue lq{leafq + threadIdx.x, 128};
-    enum { X0 = 0, X1, X2, D0, D1, D2, SS, PP };
-    int err = 0;
-    int stack[kStackSize];
-    int hits[kMaxHits];
-    const int lane = threadIdx.x & 31;
-    // warp-uniform loop over groups of 32 consecutive walks
-    for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); base < total;
-         base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t idx = base + lane;
-        const bool live = idx < total;
-        const int64_t qi = live ? idx / p.N : 0;
-        const int64_t wi = idx - qi * p.N;
-        double value = 0.0;
-        if (live) {
-            const uint32_t q = p.q_base + (uint32_t)qi;
-            const uint32_t w = (uint32_t)(p.walk_begin + wi);
-            ws.set(X0, pack_ff({p.queries[3 * qi], 0.f}));
-            ws.set(X1, pack_ff({p.queries[3 * qi + 1], 0.f}));
-            ws.set(X2, pack_ff({p.queries[3 * qi + 2], 0.f}));
-            ws.set(SS, 0.0);
-            ws.set(PP, 1.0);
-            const LineOut lo{DEBUG && p.line_m ? p.line_m + idx * p.M : nullptr,
-                             DEBUG && p.line_prim ? p.line_prim + idx * p.M : nullptr,
-                             DEBUG && p.line_flag ? p.line_flag + idx * p.M : nullptr};
-            if (DEBUG)
-                for (int k = 0; k < p.M; ++k) lo.put(k, -1, -1, 0);
-            int self = -1, k0 = 0, wflag = 0;
-            if (p.query_prim) {
-                const int32_t prim = p.query_prim[qi];
-                if (prim >= 0 && prim < p.T) {
-                    self = p.inv_order[prim];
-                    k0 = 1;
-                }
+struct NdWalks : WalkTiles {
+    using Base = WalkTiles;
+    using Base::p;
+    __device__ __forceinline__ explicit NdWalks(const WalkParams& p_) : Base(p_) {}
+    template <class Mem>
+    __device__ __forceinline__ void begin(const Mem& mem, LaneWalk& lw)
+    {
+        float3 x;
+        const int64_t qi = Base::start(mem, lw, x);
+        mem.set_x(0, {x.x, 0.f});
+        mem.set_x(1, {x.y, 0.f});
+        mem.set_x(2, {x.z, 0.f});
+        mem.set(kAccS, 0.0);
+        mem.set(kAccP, 1.0);
+        lw.self = -1;
+        lw.k = 0;
+        lw.flag = 0;
+        if (p.query_prim) {
+            const int32_t prim = p.query_prim[qi];
+            if (prim >= 0 && prim < p.T) {
+                lw.self = p.inv_order[prim];
+                lw.k = 1;
             }
-            for (int k = k0; k <= p.M; ++k) {
-                // source at vertex k
-                {
-                    FFPoint y;
-                    float b0, b1, b2;
-                    const int64_t j = area_sample_ff(p, key, q, w, (uint32_t)k, y, b0, b1, b2);
-                    float r2 = 0.f;
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        const ff x = unpack_ff(ws.get(X0 + c));
-                        const float rc = ff_add(ff_sub({y.v0[c], 0.f}, x), y.p[c]).hi;
-                        r2 = __fmaf_rn(rc, rc, r2);
-                    }
-                    if (r2 >= rmin2) {
-                        const float f = sl_data_ff(p, j, y, b0, b1, b2, WOB_BC_NEUMANN);
-                        float c = (k == 0) ? phi_f : 2.f * phi_f;
-                        if (k == p.M) c *= 0.5f;
-                        const float G = 0.0795774715459476678f * rsqrt_ftz(r2);
-                        ws.set(SS, fma(ws.get(PP), (double)(c * area_f * G * f), ws.get(SS)));
-                    }
-                }
-                if (k == p.M) break;
-                // line from vertex k to vertex k + 1
-                LinePre L;
-                {
-                    ff d[3];
-                    line_axis_ff(key, q, w, (uint32_t)k, d);
-                    ws.set(D0, pack_ff(d[0]));
-                    ws.set(D1, pack_ff(d[1]));
-                    ws.set(D2, pack_ff(d[2]));
-                    L = line_pre(make_float3(unpack_ff(ws.get(X0)).hi, unpack_ff(ws.get(X1)).hi,
-                                             unpack_ff(ws.get(X2)).hi),
-                                 make_float3(d[0].hi, d[1].hi, d[2].hi));
-                }
-                const float Tthr = p.edge_thr_L * fabsf(L.Sz);
-                Trav t;
-                trav_init(t);
-                uint32_t nn = 0, nt = 0;
-                trace_wide_q<false, false, true>(p.nodes, p.tv, L, make_float3(0.f, 0.f, 0.f), Tthr, p.tauL,
-                                           p.graze, self, t, hits, stack, key, q, w, (uint32_t)k, nn,
-                                           nt, err, p.iter_limit, lq);
-                wflag |= t.flag;
-                if (t.m == 0) {
-                    if (DEBUG) lo.put(k, 0, -1, t.flag);
-                    break;
-                }
-                const int pos = select_hit(p.tv, t, hits, key, q, w, (uint32_t)k);
-                if (DEBUG) lo.put(k, t.m, (int)prim_of(p.tv, pos), t.flag);
-                const ff x[3] = {unpack_ff(ws.get(X0)), unpack_ff(ws.get(X1)), unpack_ff(ws.get(X2))};
-                const ff d[3] = {unpack_ff(ws.get(D0)), unpack_ff(ws.get(D1)), unpack_ff(ws.get(D2))};
-                ff y[3];
-                const double ms = (double)(t.m * refine_hit_ff(p.tv, pos, x, d, y));
-                ws.set(PP, ws.get(PP) * ((k == 0) ? 0.5 * phi * ms : phi * ms));
-                ws.set(X0, pack_ff(y[0]));
-                ws.set(X1, pack_ff(y[1]));
-                ws.set(X2, pack_ff(y[2]));
-                self = pos;
-            }
-            value = ws.get(SS);
-            if (p.per_walk) p.per_walk[idx] = value;
-            if (DEBUG && p.walk_flag) p.walk_flag[idx] = (uint8_t)wflag;
         }
-        if (p.part) add_tile_partials(value, live, qi, wi, p.tpq, p.part);
+        if (DEBUG) {
+            const LineOut lo = Base::lines(lw);
+            for (int k = 0; k < p.M; ++k) lo.put(k, -1, -1, 0);
+        }
     }
+    // source at vertex k
+    template <class Mem>
+    __device__ __forceinline__ bool depart(const Mem& mem, const LaneWalk& lw) const
+    {
+        FFPoint y;
+        float b0, b1, b2;
+        const int64_t j = area_sample_ff(p, Base::key(lw), mem.q(), mem.w(), (uint32_t)lw.k, y, b0,
+                                         b1, b2);
+        float r2 = 0.f;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const float rc = ff_add(ff_sub({y.v0[c], 0.f}, mem.x(c)), y.p[c]).hi;
+            r2 = __fmaf_rn(rc, rc, r2);
+        }
+        const float rmin2 = (float)(1e-24 * p.L * p.L);
+        if (r2 >= rmin2) {
+            const float f = sl_data_ff(p, j, y, b0, b1, b2, WOB_BC_NEUMANN);
+            float c = (lw.k == 0) ? (float)p.phi : 2.f * (float)p.phi;
+            if (lw.k == p.M) c *= 0.5f;
+            const float G = 0.0795774715459476678f * rsqrt_ftz(r2);
+            mem.set(kAccS, fma(mem.get(kAccP), (double)(c * (float)p.area * G * f), mem.get(kAccS)));
+        }
+        return lw.k < p.M;
+    }
+    // line from vertex k to vertex k + 1
+    template <class Mem>
+    __device__ __forceinline__ bool land(const Mem& mem, LaneWalk& lw, int m, int pos, int flag)
+    {
+        if (DEBUG) {
+            lw.flag |= flag;
+            Base::lines(lw).put(lw.k, m, pos >= 0 ? (int)prim_of(p.tv, pos) : -1, flag);
+        }
+        if (m == 0) return false;
+        const double phi = (double)p.phi;
+        const ff x[3] = {mem.x(0), mem.x(1), mem.x(2)};
+        const ff d[3] = {mem.d(0), mem.d(1), mem.d(2)};
+        ff y[3];
+        const double ms = (double)(m * refine_hit_ff(p.tv, pos, x, d, y));
+        mem.set(kAccP, mem.get(kAccP) * ((lw.k == 0) ? 0.5 * phi * ms : phi * ms));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) mem.set_x(c, y[c]);
+        lw.self = pos;
+        ++lw.k;
+        return true;
+    }
+    template <class Mem>
+    __device__ __forceinline__ double value(const Mem& mem, const LaneWalk& lw) const
+    {
+        const double v = mem.get(kAccS);
+        if (DEBUG) {
+            const int64_t idx = Base::index(lw);
+            if (p.per_walk) p.per_walk[idx] = v;
+            if (p.walk_flag) p.walk_flag[idx] = (uint8_t)lw.flag;
+        }
+        return v;
+    }
+};
+
+template <bool DEBUG>
+__global__ void __launch_bounds__(kLineThreads, DEBUG ? kDebugBlocks : kNdBlocks) k_nd_lines(WalkParams p)
+{
+    __shared__ LineShared sm;
+    extern __shared__ int line_stack[];
+    int err = 0;
+    WalkCount c{0, 0, 0, 0, 0};
+    NdWalks<DEBUG> pol(p);
+    run_lines<NdWalks<DEBUG>, false>(pol, sm.lane(line_stack), sm.vals, p.stack_levels, err, c);
+    if (err) atomicOr(p.error_word, err);
+}
+
+__global__ void __launch_bounds__(kGroupThreads, kGroupBlocks) k_nd_groups(WalkParams p)
+{
+    __shared__ GroupShared sm;
+    extern __shared__ int line_stack[];
+    int err = 0;
+    NdWalks<false> pol(p);
+    run_line_groups(pol, sm, line_stack, p.stack_levels, err);
     if (err) atomicOr(p.error_word, err);
 }
 
@@ -734,27 +854,29 @@ __global__ void k_fwd_mix(WalkParams p, const double* __restrict__ aq_incl, doub
     }
 }
 
-__global__ void __launch_bounds__(128, WOB_DL_MIN_BLOCKS)
-    k_fwd_paths(WalkParams p, int64_t n_paths, int start_mode, const double* __restrict__ wcdf,
-                double* __restrict__ zpos, double* __restrict__ zw, uint8_t* __restrict__ flags)
-{
-    const StreamKey key{p.key0, p.key1};
-    const double phi = (double)p.phi;
-    const double* cdf = start_mode == 1 ? wcdf : p.cdf;
-    const double tot = start_mode == 1 ? wcdf[p.T - 1] : p.area;
-    int err = 0;
-    int stack[kStackSize];
-    int hits[kMaxHits];
-    for (int64_t path = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; path < n_paths;
-         path += (int64_t)gridDim.x * blockDim.x) {
-        double* zp = zpos + path * p.M * 3;
-        double* wp = zw + path * p.M;
-        for (int j = 0; j < p.M; ++j) {
-            zp[3 * j] = zp[3 * j + 1] = zp[3 * j + 2] = 0.0;
-            wp[j] = 0.0;
-        }
-        const uint32_t q = (uint32_t)path;
-        const u32x4 u = stream_block(key, q, kForwardWalk, 0u, kPurposeArea, 0u, 0u);
+// The paths as the line engine's walks (p.Q x p.N = paths): a path's weight
+// a_j waits in the first accumulator, its vertices and weights go to zpos
+// and zw.
+struct FwdPaths : WalkTiles {
+    using Base = WalkTiles;
+    using Base::p;
+    int start_mode;
+    const double* wcdf;
+    double *zpos, *zw;
+    uint8_t* flags;
+    __device__ __forceinline__ FwdPaths(const WalkParams& p_, int start_mode_, const double* wcdf_,
+                                        double* zpos_, double* zw_, uint8_t* flags_)
+        : Base(p_), start_mode(start_mode_), wcdf(wcdf_), zpos(zpos_), zw(zw_), flags(flags_)
+    {
+    }
+    template <class Mem>
+    __device__ __forceinline__ void begin(const Mem& mem, LaneWalk& lw)
+    {
+        const double* cdf = start_mode == 1 ? wcdf : p.cdf;
+        const double tot = start_mode == 1 ? wcdf[p.T - 1] : p.area;
+        const uint32_t q = (uint32_t)Base::index(lw);
+        mem.set_ids(q, kForwardWalk);
+        const u32x4 u = stream_block(Base::key(lw), q, kForwardWalk, 0u, kPurposeArea, 0u, 0u);
         const long long target = __double_as_longlong(u53(u.x, u.y) * tot);
         int64_t lo = 0, hi = p.T - 1;
         while (lo < hi) {
@@ -767,39 +889,80 @@ __global__ void __launch_bounds__(128, WOB_DL_MIN_BLOCKS)
         const double pdf = start_mode == 1
                                ? ((cdf[lo] - (lo > 0 ? cdf[lo - 1] : 0.0)) / p.tri_n[lo].area) / tot
                                : 1.0 / p.area;
-        double a = 2.0 * phi * (double)sl_data_ff(p, lo, y, b0, b1, b2, WOB_BC_NEUMANN, true) / pdf;
-        ff z[3];
+        mem.set(kAccS, 2.0 * (double)p.phi *
+                           (double)sl_data_ff(p, lo, y, b0, b1, b2, WOB_BC_NEUMANN, true) / pdf);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) z[c] = ff_add({y.v0[c], 0.f}, y.p[c]);
-        int self = p.inv_order[lo], flag = 0;
-        for (int j = 0; j < p.M; ++j) {
-            zp[3 * j] = ff_join(z[0]);
-            zp[3 * j + 1] = ff_join(z[1]);
-            zp[3 * j + 2] = ff_join(z[2]);
-            wp[j] = (j == p.M - 1 ? 0.5 : 1.0) * a;
-            if (j == p.M - 1) break;
-            ff d[3];
-            line_axis_ff(key, q, kForwardWalk, (uint32_t)j, d);
-            const LinePre L = line_pre(make_float3(z[0].hi, z[1].hi, z[2].hi),
-                                       make_float3(d[0].hi, d[1].hi, d[2].hi));
-            const float Tthr = p.edge_thr_L * fabsf(L.Sz);
-            Trav tr;
-            trav_init(tr);
-            uint32_t nn = 0, nt = 0;
-            trace_wide<false, false>(p.nodes, p.tv, L, make_float3(0.f, 0.f, 0.f), Tthr, p.tauL,
-                                     p.graze, self, tr, hits, stack, key, q, kForwardWalk,
-                                     (uint32_t)j, nn, nt, err, p.iter_limit);
-            flag |= tr.flag;
-            if (tr.m == 0) break;
-            const int pos = select_hit(p.tv, tr, hits, key, q, kForwardWalk, (uint32_t)j);
-            ff yz[3];
-            a *= phi * (double)(tr.m * refine_hit_ff(p.tv, pos, z, d, yz));
-#pragma unroll
-            for (int c = 0; c < 3; ++c) z[c] = yz[c];
-            self = pos;
-        }
-        if (flags) flags[path] = (uint8_t)flag;
+        for (int c = 0; c < 3; ++c) mem.set_x(c, ff_add({y.v0[c], 0.f}, y.p[c]));
+        lw.self = p.inv_order[lo];
+        lw.k = 0;
+        lw.flag = 0;
     }
+    __device__ __forceinline__ void put(const LaneWalk& lw, int j, ff x, ff y, ff z, double w) const
+    {
+        const int64_t r = Base::index(lw) * p.M + j;
+        zpos[3 * r] = ff_join(x);
+        zpos[3 * r + 1] = ff_join(y);
+        zpos[3 * r + 2] = ff_join(z);
+        zw[r] = w;
+    }
+    template <class Mem>
+    __device__ __forceinline__ bool depart(const Mem& mem, const LaneWalk& lw) const
+    {
+        const double a = mem.get(kAccS);
+        const bool last = lw.k == p.M - 1;
+        put(lw, lw.k, mem.x(0), mem.x(1), mem.x(2), last ? 0.5 * a : a);
+        return !last;
+    }
+    template <class Mem>
+    __device__ __forceinline__ bool land(const Mem& mem, LaneWalk& lw, int m, int pos, int flag)
+    {
+        lw.flag |= flag;
+        if (m == 0) return false;
+        const ff x[3] = {mem.x(0), mem.x(1), mem.x(2)};
+        const ff d[3] = {mem.d(0), mem.d(1), mem.d(2)};
+        ff y[3];
+        const int s = refine_hit_ff(p.tv, pos, x, d, y);
+        mem.set(kAccS, mem.get(kAccS) * ((double)p.phi * (double)(m * s)));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) mem.set_x(c, y[c]);
+        lw.self = pos;
+        ++lw.k;
+        return true;
+    }
+    // a path that a missed line ended: its remaining records are zero
+    template <class Mem>
+    __device__ __forceinline__ double value(const Mem&, const LaneWalk& lw) const
+    {
+        const ff zero = {0.f, 0.f};
+        for (int j = lw.k + 1; j < p.M; ++j) put(lw, j, zero, zero, zero, 0.0);
+        if (flags) flags[Base::index(lw)] = (uint8_t)lw.flag;
+        return 0.0;
+    }
+    __device__ __forceinline__ void close(int, int, double) const {}
+};
+
+__global__ void __launch_bounds__(kLineThreads, kLineBlocks - 1)
+    k_fwd_lines(WalkParams p, int start_mode, const double* __restrict__ wcdf,
+                double* __restrict__ zpos, double* __restrict__ zw, uint8_t* __restrict__ flags)
+{
+    __shared__ LineShared sm;
+    extern __shared__ int line_stack[];
+    int err = 0;
+    WalkCount c{0, 0, 0, 0, 0};
+    FwdPaths pol(p, start_mode, wcdf, zpos, zw, flags);
+    run_lines<FwdPaths, false>(pol, sm.lane(line_stack), sm.vals, p.stack_levels, err, c);
+    if (err) atomicOr(p.error_word, err);
+}
+
+__global__ void __launch_bounds__(kGroupThreads, kGroupBlocks)
+    k_fwd_groups(WalkParams p, int start_mode, const double* __restrict__ wcdf,
+                 double* __restrict__ zpos, double* __restrict__ zw, uint8_t* __restrict__ flags)
+{
+    __shared__ GroupShared sm;
+    extern __shared__ int line_stack[];
+    int err = 0;
+    FwdPaths pol(p, start_mode, wcdf, zpos, zw, flags);
+    run_line_groups(pol, sm, line_stack, p.stack_levels, err);
     if (err) atomicOr(p.error_word, err);
 }
 
@@ -1158,25 +1321,53 @@ __global__ void k_philox(const uint32_t* __restrict__ ctr, const uint32_t* __res
 
 }  // namespace
 
-int launch_dl_walks(const WalkParams& p, bool counted, bool debug, cudaStream_t s)
+namespace {
+
+// Launch a line-walk kernel (one lane per walk) with its traversal stacks in
+// dynamic shared memory.
+template <class K, class... Args>
+int launch_lines(K kernel, const WalkParams& p, cudaStream_t s, Args... args)
 {
-    const int threads = 128;
-    const int64_t work = p.Q * (int64_t)p.N;
-    if (p.per_walk_grad) {
-        k_dl_walks<false, false, true><<<grid_for((const void*)k_dl_walks<false, false, true>,
-                                                  threads, 0, work), threads, 0, s>>>(p);
-    } else if (counted) {
-        k_dl_walks<true, true><<<grid_for((const void*)k_dl_walks<true, true>, threads, 0, work),
-                                 threads, 0, s>>>(p);
-    } else if (debug) {
-        k_dl_walks<false, true><<<grid_for((const void*)k_dl_walks<false, true>, threads, 0, work),
-                                  threads, 0, s>>>(p);
-    } else {
-        k_dl_walks<false, false><<<grid_for((const void*)k_dl_walks<false, false>, threads, 0, work),
-                                   threads, 0, s>>>(p);
-    }
+    size_t smem = 0;
+    WOB_TRY(line_stack_bytes((const void*)kernel, p.stack_levels * kLineThreads, smem));
+    kernel<<<grid_for((const void*)kernel, kLineThreads, smem, p.Q * (int64_t)p.N), kLineThreads,
+             smem, s>>>(p, args...);
     WOB_CUDA_TRY(cudaGetLastError());
     return WOB_OK;
+}
+
+// The same for its form with kG lanes per walk.
+template <class K, class... Args>
+int launch_groups(K kernel, const WalkParams& p, cudaStream_t s, Args... args)
+{
+    size_t smem = 0;
+    WOB_TRY(line_stack_bytes((const void*)kernel, p.stack_levels * kGroups, smem));
+    kernel<<<grid_for((const void*)kernel, kGroupThreads, smem, kG * p.Q * (int64_t)p.N),
+             kGroupThreads, smem, s>>>(p, args...);
+    WOB_CUDA_TRY(cudaGetLastError());
+    return WOB_OK;
+}
+
+// Too few walks to fill the GPU one lane each.
+bool few_walks(const WalkParams& p)
+{
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return p.Q * (int64_t)p.N <= sms * kGroupWalksPerSm;
+}
+
+}  // namespace
+
+int launch_dl_walks(const WalkParams& p, bool counted, bool debug, cudaStream_t s)
+{
+    if (p.per_walk_grad)
+        return few_walks(p) ? launch_groups(k_dl_groups<true>, p, s)
+                            : launch_lines(k_dl_lines<false, false, true>, p, s);
+    if (counted) return launch_lines(k_dl_lines<true, true, false>, p, s);
+    if (debug) return launch_lines(k_dl_lines<false, true, false>, p, s);
+    return few_walks(p) ? launch_groups(k_dl_groups<false>, p, s)
+                        : launch_lines(k_dl_lines<false, false, false>, p, s);
 }
 
 int launch_sl_walks(const WalkParams& p, bool debug, cudaStream_t s)
@@ -1199,14 +1390,8 @@ int launch_sl_walks(const WalkParams& p, bool debug, cudaStream_t s)
 
 int launch_nd_walks(const WalkParams& p, bool debug, cudaStream_t s)
 {
-    const int threads = 128;
-    const int64_t work = p.Q * (int64_t)p.N;
-    if (debug)
-        k_nd_walks<true><<<grid_for((const void*)k_nd_walks<true>, threads, 0, work), threads, 0, s>>>(p);
-    else
-        k_nd_walks<false><<<grid_for((const void*)k_nd_walks<false>, threads, 0, work), threads, 0, s>>>(p);
-    WOB_CUDA_TRY(cudaGetLastError());
-    return WOB_OK;
+    if (debug) return launch_lines(k_nd_lines<true>, p, s);
+    return few_walks(p) ? launch_groups(k_nd_groups, p, s) : launch_lines(k_nd_lines<false>, p, s);
 }
 
 int launch_forward(const WalkParams& p, int64_t n_paths, int start_mode, double beta,
@@ -1229,9 +1414,12 @@ int launch_forward(const WalkParams& p, int64_t n_paths, int start_mode, double 
         }
     }
     const int threads = 128;
-    k_fwd_paths<<<grid_for((const void*)k_fwd_paths, threads, 0, n_paths), threads, 0, s>>>(
-        p, n_paths, start_mode, buf ? buf + 3 * p.T : nullptr, zpos, zw, flags);
-    int rc = cudaGetLastError() == cudaSuccess ? WOB_OK : WOB_ERR_CUDA;
+    WalkParams pp = p;  // the paths as the engine's walks
+    pp.Q = 1;
+    pp.N = (int32_t)n_paths;
+    const double* start_cdf = buf ? buf + 3 * p.T : nullptr;
+    int rc = few_walks(pp) ? launch_groups(k_fwd_groups, pp, s, start_mode, start_cdf, zpos, zw, flags)
+                           : launch_lines(k_fwd_lines, pp, s, start_mode, start_cdf, zpos, zw, flags);
     if (buf) cudaFreeAsync(buf, s);
     if (rc == WOB_OK && Q > 0) {
         // packed records and live bytes, then (sum, sum of squares) per split and query

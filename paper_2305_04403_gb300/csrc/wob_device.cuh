@@ -163,13 +163,17 @@ __device__ __forceinline__ void line_axis_ff(StreamKey key, uint32_t q, uint32_t
 __device__ __forceinline__ int leaf_first(int ref) { return (~ref) >> 3; }
 __device__ __forceinline__ int leaf_count(int ref) { return ((~ref) & 7) + 1; }
 
-struct LinePre {
-    float ox, oy, oz;     // origin
-    float ix, iy, iz;     // 1 / d (guarded)
-    float oix, oiy, oiz;  // o / d
-    // Woop-Benthin-Wald watertight shear
+// A line in the sheared frame of the triangle test (Woop, Benthin and Wald).
+struct LineShear {
+    float ox, oy, oz;  // origin
     int kx, ky, kz;
     float Sx, Sy, Sz;  // shear; |Sz| = 1 / |d_kz|
+};
+
+// The same line with the slab parameters of the box test.
+struct LinePre : LineShear {
+    float ix, iy, iz;     // 1 / d (guarded)
+    float oix, oiy, oiz;  // o / d
 };
 
 __device__ __forceinline__ float guard_inv(float d)
@@ -180,12 +184,10 @@ __device__ __forceinline__ float guard_inv(float d)
 
 __device__ __forceinline__ float comp(float3 v, int k) { return k == 0 ? v.x : (k == 1 ? v.y : v.z); }
 
-__device__ __forceinline__ LinePre line_pre(float3 o, float3 d)
+__device__ __forceinline__ LineShear line_shear(float3 o, float3 d)
 {
-    LinePre L;
+    LineShear L;
     L.ox = o.x; L.oy = o.y; L.oz = o.z;
-    L.ix = guard_inv(d.x); L.iy = guard_inv(d.y); L.iz = guard_inv(d.z);
-    L.oix = o.x * L.ix; L.oiy = o.y * L.iy; L.oiz = o.z * L.iz;
     const float ax = fabsf(d.x), ay = fabsf(d.y), az = fabsf(d.z);
     int kz = (ax > ay) ? (ax > az ? 0 : 2) : (ay > az ? 1 : 2);
     int kx = kz + 1 == 3 ? 0 : kz + 1;
@@ -199,16 +201,13 @@ __device__ __forceinline__ LinePre line_pre(float3 o, float3 d)
     return L;
 }
 
-// Does the line meet the box [lo, hi]?  No parameter range: a line.
-__device__ __forceinline__ bool line_box(const LinePre& L, float lox, float hix, float loy,
-                                         float hiy, float loz, float hiz)
+__device__ __forceinline__ LinePre line_pre(float3 o, float3 d)
 {
-    const float t0x = fmaf(lox, L.ix, -L.oix), t1x = fmaf(hix, L.ix, -L.oix);
-    const float t0y = fmaf(loy, L.iy, -L.oiy), t1y = fmaf(hiy, L.iy, -L.oiy);
-    const float t0z = fmaf(loz, L.iz, -L.oiz), t1z = fmaf(hiz, L.iz, -L.oiz);
-    const float tn = fmaxf(fmaxf(fminf(t0x, t1x), fminf(t0y, t1y)), fminf(t0z, t1z));
-    const float tf = fminf(fminf(fmaxf(t0x, t1x), fmaxf(t0y, t1y)), fmaxf(t0z, t1z));
-    return tn <= tf;
+    LinePre L;
+    static_cast<LineShear&>(L) = line_shear(o, d);
+    L.ix = guard_inv(d.x); L.iy = guard_inv(d.y); L.iz = guard_inv(d.z);
+    L.oix = o.x * L.ix; L.oiy = o.y * L.iy; L.oiz = o.z * L.iz;
+    return L;
 }
 
 // ---------------------------------------------------------------------------
@@ -282,7 +281,7 @@ __device__ __forceinline__ void keep_min(uint64_t k, uint32_t prim, int pos, uin
 // opposite values for it (watertight), and the near-degenerate flag is
 // decided from the true distances of the line to the edges.
 // Sheared coordinates (kx, ky) of a point p relative to the line origin.
-__device__ __forceinline__ float2 shear_rel(const float4& p, const LinePre& L)
+__device__ __forceinline__ float2 shear_rel(const float4& p, const LineShear& L)
 {
     const float3 r = make_float3(p.x - L.ox, p.y - L.oy, p.z - L.oz);
     const float rz = comp(r, L.kz);
@@ -297,7 +296,7 @@ __device__ __forceinline__ float2 shear_rel(const float4& p, const LinePre& L)
 // len2 receives |d x e|^2 / d_kz^2, so that f^2 / len2 is the squared
 // distance of the line to the edge's supporting line.
 __device__ __forceinline__ float edge_fn(const float4& P, float2 Pp, const float4& Q, float2 Qp,
-                                         const LinePre& L, float& len2)
+                                         const LineShear& L, float& len2)
 {
     const float3 e = make_float3(Q.x - P.x, Q.y - P.y, Q.z - P.z);
     const float ez = comp(e, L.kz);
@@ -321,7 +320,7 @@ struct EdgeFns {
     int flag;
 };
 
-static __device__ __noinline__ EdgeFns near_edges(float4 a4, float4 b4, float4 c4, LinePre L, float tauL)
+static __device__ __noinline__ EdgeFns near_edges(float4 a4, float4 b4, float4 c4, LineShear L, float tauL)
 {
     const float2 A = shear_rel(a4, L), B = shear_rel(b4, L), C = shear_rel(c4, L);
     float lu, lv, lw;
@@ -337,7 +336,7 @@ static __device__ __noinline__ EdgeFns near_edges(float4 a4, float4 b4, float4 c
 }
 
 __device__ __forceinline__ bool line_tri(const float4& a4, const float4& b4, const float4& c4,
-                                         const LinePre& L, float Trare, float tauL, float graze,
+                                         const LineShear& L, float Trare, float tauL, float graze,
                                          int& flag, float& tl)
 {
     const float3 A = make_float3(a4.x - L.ox, a4.y - L.oy, a4.z - L.oz);
@@ -428,6 +427,77 @@ __device__ __forceinline__ float dequant(uint32_t w, int b)
     return __uint_as_float(__byte_perm(w, 0x3F800000u, 0x7604u | ((uint32_t)b << 4)));
 }
 
+// The children of a wide node that a line meets, as a mask of slots: header h
+// (f[0]), quantised planes qx, qy, qz (f[1..3]), slab values of the line.
+__device__ __forceinline__ uint32_t node_hits(float4 h, uint4 qx, uint4 qy, uint4 qz, float ix,
+                                              float iy, float iz, float oix, float oiy, float oiz)
+{
+    const uint32_t hdr = __float_as_uint(h.w);
+    const int nch = hdr >> 28;
+    // slab parameter of a quantised plane: (origin + q s - o) / d
+    // = (1 + q 2^-15) a + b with a = 2^15 s / d (see dequant)
+    const float ax = __uint_as_float(((hdr & 255u) + 15u) << 23) * ix;
+    const float ay = __uint_as_float((((hdr >> 8) & 255u) + 15u) << 23) * iy;
+    const float az = __uint_as_float((((hdr >> 16) & 255u) + 15u) << 23) * iz;
+    const float bx = fmaf(h.x, ix, -oix) - ax, by = fmaf(h.y, iy, -oiy) - ay,
+                bz = fmaf(h.z, iz, -oiz) - az;
+    // per axis the near plane is the low one when the axis component
+    // is positive (t = q a + b is monotone in q): pick near / far
+    // byte words once, so a slab test is max of 3 nears <= min of 3 fars
+    const bool px_ = ix >= 0.f, py_ = iy >= 0.f, pz_ = iz >= 0.f;
+    const uint32_t nx0 = px_ ? qx.x : qx.z, nx1 = px_ ? qx.y : qx.w;
+    const uint32_t fx0 = px_ ? qx.z : qx.x, fx1 = px_ ? qx.w : qx.y;
+    const uint32_t ny0 = py_ ? qy.x : qy.z, ny1 = py_ ? qy.y : qy.w;
+    const uint32_t fy0 = py_ ? qy.z : qy.x, fy1 = py_ ? qy.w : qy.y;
+    const uint32_t nz0 = pz_ ? qz.x : qz.z, nz1 = pz_ ? qz.y : qz.w;
+    const uint32_t fz0 = pz_ ? qz.z : qz.x, fz1 = pz_ ? qz.w : qz.y;
+    uint32_t hit = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const float tnx = fmaf(dequant(j < 4 ? nx0 : nx1, j & 3), ax, bx);
+        const float tfx = fmaf(dequant(j < 4 ? fx0 : fx1, j & 3), ax, bx);
+        const float tny = fmaf(dequant(j < 4 ? ny0 : ny1, j & 3), ay, by);
+        const float tfy = fmaf(dequant(j < 4 ? fy0 : fy1, j & 3), ay, by);
+        const float tnz = fmaf(dequant(j < 4 ? nz0 : nz1, j & 3), az, bz);
+        const float tfz = fmaf(dequant(j < 4 ? fz0 : fz1, j & 3), az, bz);
+        const float tn = fmaxf(fmaxf(tnx, tny), tnz);
+        const float tf = fminf(fminf(tfx, tfy), tfz);
+        hit |= (tn <= tf ? 1u : 0u) << j;
+    }
+    return hit & ((1u << nch) - 1u);
+}
+
+// The same test of the children j, j + G, ... only (bit i of the result:
+// child j + G i), for G lanes that share a line.
+template <int G>
+__device__ __forceinline__ uint32_t lane_children(float4 h, uint4 qx, uint4 qy, uint4 qz, int j, float ix,
+                                                  float iy, float iz, float oix, float oiy, float oiz)
+{
+    const uint32_t hdr = __float_as_uint(h.w);
+    const int nch = hdr >> 28;
+    const float ax = __uint_as_float(((hdr & 255u) + 15u) << 23) * ix;
+    const float ay = __uint_as_float((((hdr >> 8) & 255u) + 15u) << 23) * iy;
+    const float az = __uint_as_float((((hdr >> 16) & 255u) + 15u) << 23) * iz;
+    const float bx = fmaf(h.x, ix, -oix) - ax, by = fmaf(h.y, iy, -oiy) - ay,
+                bz = fmaf(h.z, iz, -oiz) - az;
+    uint32_t hit = 0;
+#pragma unroll
+    for (int i = 0; i < 8 / G; ++i) {
+        const bool upper = G == 8 ? j >= 4 : ((G * i) >> 2) != 0;  // word of the child's bytes
+        const uint32_t sel = 0x7604u | ((uint32_t)((j + G * i) & 3) << 4);
+        auto plane = [&](uint32_t w0, uint32_t w1, float a, float b) {
+            return fmaf(__uint_as_float(__byte_perm(upper ? w1 : w0, 0x3F800000u, sel)), a, b);
+        };
+        const float x0 = plane(qx.x, qx.y, ax, bx), x1 = plane(qx.z, qx.w, ax, bx);
+        const float y0 = plane(qy.x, qy.y, ay, by), y1 = plane(qy.z, qy.w, ay, by);
+        const float z0 = plane(qz.x, qz.y, az, bz), z1 = plane(qz.z, qz.w, az, bz);
+        const float tn = fmaxf(fmaxf(fminf(x0, x1), fminf(y0, y1)), fminf(z0, z1));
+        const float tf = fminf(fminf(fmaxf(x0, x1), fmaxf(y0, y1)), fmaxf(z0, z1));
+        hit |= (j + G * i < nch && tn <= tf ? 1u : 0u) << i;
+    }
+    return hit;
+}
+
 __device__ __forceinline__ int pick4(int4 v, int j)
 {
     return j == 0 ? v.x : (j == 1 ? v.y : (j == 2 ? v.z : v.w));
@@ -456,13 +526,7 @@ struct LeafQueue {
     __device__ __forceinline__ int& operator[](int i) const { return base[i * stride]; }
 };
 
-// HIT_MASK picks how the slots beyond a node's children are dropped: one
-// mask per node (true) or a test per slot (false).  Both give the same hit
-// set; which runs faster depends on the kernel's register allocation (on a
-// GB300 the mask is 4% faster in the direct-BIE walk kernel, 3% in the
-// batched one, 1% in the gradient walks and 1% slower in the plain
-// double-layer walks).
-template <bool COUNT, bool SUM_S, bool HIT_MASK = false>
+template <bool COUNT, bool SUM_S>
 __device__ __forceinline__ void trace_wide_q(const float4* __restrict__ wn,
                                              const float4* __restrict__ tv, const LinePre& L,
                                              float3 d, float Tthr, float tauL, float graze,
@@ -497,43 +561,11 @@ __device__ __forceinline__ void trace_wide_q(const float4* __restrict__ wn,
             if (COUNT) n_nodes++;
             const float4* nd = wn + 6 * node;
             const float4 h = __ldg(nd);
-            const uint32_t hdr = __float_as_uint(h.w);
-            const int nint = (hdr >> 24) & 15, nch = hdr >> 28;
-            // slab parameter of a quantised plane: (origin + q s - o) / d
-            // = (1 + q 2^-15) a + b with a = 2^15 s / d (see dequant)
-            const float ax = __uint_as_float(((hdr & 255u) + 15u) << 23) * L.ix;
-            const float ay = __uint_as_float((((hdr >> 8) & 255u) + 15u) << 23) * L.iy;
-            const float az = __uint_as_float((((hdr >> 16) & 255u) + 15u) << 23) * L.iz;
-            const float bx = fmaf(h.x, L.ix, -L.oix) - ax, by = fmaf(h.y, L.iy, -L.oiy) - ay,
-                        bz = fmaf(h.z, L.iz, -L.oiz) - az;
+            const int nint = (__float_as_uint(h.w) >> 24) & 15;
             const uint4 qx = __ldg(reinterpret_cast<const uint4*>(nd + 1));
             const uint4 qy = __ldg(reinterpret_cast<const uint4*>(nd + 2));
             const uint4 qz = __ldg(reinterpret_cast<const uint4*>(nd + 3));
-            // per axis the near plane is the low one when the axis component
-            // is positive (t = q a + b is monotone in q): pick near / far
-            // byte words once, so a slab test is max of 3 nears <= min of 3 fars
-            const bool px_ = L.ix >= 0.f, py_ = L.iy >= 0.f, pz_ = L.iz >= 0.f;
-            const uint32_t nx0 = px_ ? qx.x : qx.z, nx1 = px_ ? qx.y : qx.w;
-            const uint32_t fx0 = px_ ? qx.z : qx.x, fx1 = px_ ? qx.w : qx.y;
-            const uint32_t ny0 = py_ ? qy.x : qy.z, ny1 = py_ ? qy.y : qy.w;
-            const uint32_t fy0 = py_ ? qy.z : qy.x, fy1 = py_ ? qy.w : qy.y;
-            const uint32_t nz0 = pz_ ? qz.x : qz.z, nz1 = pz_ ? qz.y : qz.w;
-            const uint32_t fz0 = pz_ ? qz.z : qz.x, fz1 = pz_ ? qz.w : qz.y;
-            uint32_t hit = 0;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const float tnx = fmaf(dequant(j < 4 ? nx0 : nx1, j & 3), ax, bx);
-                const float tfx = fmaf(dequant(j < 4 ? fx0 : fx1, j & 3), ax, bx);
-                const float tny = fmaf(dequant(j < 4 ? ny0 : ny1, j & 3), ay, by);
-                const float tfy = fmaf(dequant(j < 4 ? fy0 : fy1, j & 3), ay, by);
-                const float tnz = fmaf(dequant(j < 4 ? nz0 : nz1, j & 3), az, bz);
-                const float tfz = fmaf(dequant(j < 4 ? fz0 : fz1, j & 3), az, bz);
-                const float tn = fmaxf(fmaxf(tnx, tny), tnz);
-                const float tf = fminf(fminf(tfx, tfy), tfz);
-                if (HIT_MASK) hit |= (tn <= tf ? 1u : 0u) << j;
-                else if (j < nch && tn <= tf) hit |= 1u << j;
-            }
-            if (HIT_MASK) hit &= (1u << nch) - 1u;
+            const uint32_t hit = node_hits(h, qx, qy, qz, L.ix, L.iy, L.iz, L.oix, L.oiy, L.oiz);
             const int4 r0 = __ldg(reinterpret_cast<const int4*>(nd + 4));
             uint32_t lm = hit >> nint;  // leaf children: queue their triangles
             if (lm) {
@@ -737,42 +769,8 @@ __device__ __forceinline__ float dl_data(const DataDev& D, const float4* __restr
     return dl_data_f(D, tv, pos, make_float3((float)yd.x, (float)yd.y, (float)yd.z));
 }
 
-// Geometry a double-layer walk needs.
-struct DLGeom {
-    const float4* nodes;  // 8-wide nodes, root = node 0
-    const float4* tv;
-    int iter_limit;
-    float edge_thr_L;
-    float tauL;
-    float graze;
-};
-
 struct WalkCount {
     unsigned long long lines, nodes, tris, hits, flag;
-};
-
-// Where a walk keeps its state (point and axis as float-float pairs, S and
-// P in FP64) while its lines are traversed: eight 8-byte slots per thread in
-// shared memory, structure of arrays
-// (field j of thread t at base[j * stride + t]) so that a warp's accesses
-// are conflict-free.  The state is touched once per line; keeping it out of
-// registers leaves the traversal loop its 64 registers.
-// A float-float value in one double-sized slot (the two floats' bits, no
-// arithmetic).
-__device__ __forceinline__ double pack_ff(ff v)
-{
-    return __hiloint2double(__float_as_int(v.hi), __float_as_int(v.lo));
-}
-__device__ __forceinline__ ff unpack_ff(double v)
-{
-    return {__int_as_float(__double2hiint(v)), __int_as_float(__double2loint(v))};
-}
-
-struct WalkSlot {
-    volatile double* base;  // &smem[threadIdx.x]
-    int stride;             // threads per block
-    __device__ __forceinline__ double get(int j) const { return base[j * stride]; }
-    __device__ __forceinline__ void set(int j, double v) const { base[j * stride] = v; }
 };
 
 // Gradient weight of the first step (Sec. 4.1.3): the first line's weight
@@ -818,103 +816,6 @@ struct LineOut {
         if (flag) flag[k] = (uint8_t)fk;
     }
 };
-
-// One double-layer walk from x (Sec. 4.1.1-4.1.2, ray sampling of Sec.
-// 4.4.1): per line, draw the axis, traverse (descend to a leaf, test it,
-// repeat), pick the hit (keys only when m > 1), refine it in float-float
-// and accumulate (weight product and sum in FP64).  Returns the walk value;
-// `lo` (DEBUG only) receives the per-line outputs.  start_pos >= 0: x0 lies
-// on that triangle (leaf position) and the walk estimates the density nu(x0)
-// (Eq. indirect_double_boundary_reordered2): x0 is vertex 1 with weight 1
-// and lines 1 .. M-1 follow.  HIT_MASK: the node-test form of trace_wide_q.
-template <bool COUNT, bool DEBUG, bool GRAD = false, bool HIT_MASK = true>
-__device__ __forceinline__ double dl_walk(const DLGeom& G, const DataDev& D, double phi, int M,
-                                          StreamKey key, uint32_t q, uint32_t w, double3 x0,
-                                          int start_pos, const WalkSlot& ws, int* stack,
-                                          int* hits, int& err, int& wflag, const LineOut& lo,
-                                          WalkCount& c, LeafQueue lq)
-{
-    enum { X0 = 0, X1, X2, D0, D1, D2, SS, PP, GX, GY, GZ };  // GX..GZ: GRAD only
-    if (GRAD) {
-        ws.set(GX, 0.0);
-        ws.set(GY, 0.0);
-        ws.set(GZ, 0.0);
-    }
-    ws.set(X0, pack_ff({(float)x0.x, 0.f}));
-    ws.set(X1, pack_ff({(float)x0.y, 0.f}));
-    ws.set(X2, pack_ff({(float)x0.z, 0.f}));
-    ws.set(SS, 0.0);
-    ws.set(PP, 1.0);
-    int self = -1, k = 0;
-    if (start_pos >= 0) {
-        const double g = (double)dl_data(D, G.tv, start_pos, x0);
-        ws.set(SS, ((M == 1) ? phi : 2.0 * phi) * g);
-        self = start_pos;
-        k = 1;
-        if (DEBUG) lo.put(0, -1, -1, 0);
-    }
-    for (; k < M; ++k) {
-        LinePre L;
-        {
-            ff d[3];
-            line_axis_ff(key, q, w, (uint32_t)k, d);
-            ws.set(D0, pack_ff(d[0]));
-            ws.set(D1, pack_ff(d[1]));
-            ws.set(D2, pack_ff(d[2]));
-            L = line_pre(make_float3(unpack_ff(ws.get(X0)).hi, unpack_ff(ws.get(X1)).hi,
-                                     unpack_ff(ws.get(X2)).hi),
-                         make_float3(d[0].hi, d[1].hi, d[2].hi));
-        }
-        const float Tthr = G.edge_thr_L * fabsf(L.Sz);
-        Trav t;
-        trav_init(t);
-        uint32_t nn = 0, nt = 0;
-        trace_wide_q<COUNT, false, HIT_MASK>(G.nodes, G.tv, L, make_float3(0.f, 0.f, 0.f), Tthr,
-                                             G.tauL, G.graze, self, t, hits, stack, key, q, w, (uint32_t)k, nn, nt,
-                                   err, G.iter_limit, lq);
-        if (COUNT) {
-            c.lines++;
-            c.nodes += nn;
-            c.tris += nt;
-            c.hits += t.m;
-            c.flag += t.flag;
-        }
-        wflag |= t.flag;
-        if (t.m == 0) {
-            if (DEBUG) lo.put(k, 0, -1, t.flag);
-            ++k;
-            break;
-        }
-        const int pos = select_hit(G.tv, t, hits, key, q, w, (uint32_t)k);
-        if (DEBUG) lo.put(k, t.m, (int)prim_of(G.tv, pos), t.flag);
-        const ff x[3] = {unpack_ff(ws.get(X0)), unpack_ff(ws.get(X1)), unpack_ff(ws.get(X2))};
-        const ff d[3] = {unpack_ff(ws.get(D0)), unpack_ff(ws.get(D1)), unpack_ff(ws.get(D2))};
-        double S = ws.get(SS), P = ws.get(PP);
-        ff y[3];
-        const int sgn = refine_hit_ff(G.tv, pos, x, d, y);
-        const double ms = (double)(t.m * sgn);
-        P = (k == 0) ? 0.5 * ms : P * (-phi * ms);
-        const double g = (double)dl_data_f(D, G.tv, pos, make_float3(y[0].hi, y[1].hi, y[2].hi));
-        const double cc = (k == M - 1) ? phi : 2.0 * phi;
-        S = fma(P * cc, g, S);
-        if (GRAD && k == 0 && start_pos < 0) {
-            const double3 gf = grad_factor(G.tv, pos, make_double3((double)x[0].hi + x[0].lo, (double)x[1].hi + x[1].lo, (double)x[2].hi + x[2].lo),
-                                           make_double3((double)y[0].hi + y[0].lo, (double)y[1].hi + y[1].lo, (double)y[2].hi + y[2].lo));
-            ws.set(GX, gf.x);
-            ws.set(GY, gf.y);
-            ws.set(GZ, gf.z);
-        }
-        ws.set(X0, pack_ff(y[0]));
-        ws.set(X1, pack_ff(y[1]));
-        ws.set(X2, pack_ff(y[2]));
-        ws.set(SS, S);
-        ws.set(PP, P);
-        self = pos;
-    }
-    if (DEBUG)
-        for (int k2 = k; k2 < M; ++k2) lo.put(k2, -1, -1, 0);
-    return ws.get(SS);
-}
 
 // Per-query partial sums of the walk values.  Slot (query qi, block b of 32
 // walks of the call) holds (sum, sum of squares) at part[2 s], part[2 s + 1],

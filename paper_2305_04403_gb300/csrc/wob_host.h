@@ -39,6 +39,10 @@ void fill_params(WalkParams& p, const wob_problem* prob, const float* queries,
 // Persistent-grid size: SM count x resident blocks of `kernel` at `threads`.
 int grid_for(const void* kernel, int threads, size_t smem, int64_t work_items);
 
+// Bytes of dynamic shared memory for `entries` of the line engine's traversal
+// stacks, allowed for `kernel`.
+int line_stack_bytes(const void* kernel, int entries, size_t& bytes);
+
 // mesh.cu
 int build_mesh_impl(const float* verts, int64_t V, const int32_t* tris, int64_t T,
                     bool on_device, cudaStream_t s, MeshDev& m);

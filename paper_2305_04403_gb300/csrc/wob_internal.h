@@ -100,6 +100,7 @@ struct WalkParams {
     const float4* tv;
     const int32_t* inv_order;
     int iter_limit;  // traversal loop bound (4 x wide nodes + 64)
+    int stack_levels;  // levels of the tree: traversal stack entries per lane
     const float* verts;
     const double* verts_d;  // FP64 copy of verts (resampled area samples)
     const int32_t* tris;
