@@ -36,22 +36,37 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
 }
 
 // SiLU and its derivative with the fast exponential and reciprocal (relative
-// error ~1e-6, far below the BF16 rounding of the activations).
-__device__ __forceinline__ float silu(float a) { return __fdividef(a, 1.0f + __expf(-a)); }
+// error ~1e-6, far below the BF16 rounding of the activations).  The forms
+// that flush subnormals: 1 + e^-a and the quotient's factors are normal, and
+// the others spend two more instructions on each to handle subnormal operands.
+__device__ __forceinline__ float sigmoid(float a)
+{
+    float e, r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(a * -1.44269504f));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + e));
+    return r;
+}
+__device__ __forceinline__ float silu(float a) { return a * sigmoid(a); }
 __device__ __forceinline__ float silu_grad(float a)
 {
-    const float s = __fdividef(1.0f, 1.0f + __expf(-a));
+    const float s = sigmoid(a);
     return s * (1.0f + a * (1.0f - s));
 }
 
-// Fourier feature of column c at y: c = 32 d + 2 k + s
-__device__ __forceinline__ float feature(const float y[3], int c)
+// Twice the feature frequencies 2^(k/3), k = 0..15.
+__device__ __forceinline__ float feature_freq2(int k) { return 2.0f * exp2f((float)k * (1.0f / 3.0f)); }
+
+// The 32 features of one coordinate as 16 BF16 pairs (sin, cos) of
+// 2 pi f_k y, frequency k in word k; f2: feature_freq2(0..15), formed once
+// per block (an exponential per feature otherwise).
+__device__ __forceinline__ void features8(float y, const float* f2, uint32_t (&w)[8])
 {
-    const int d = c >> 5, j = c & 31, k = j >> 1;
-    const float f = exp2f((float)k * (1.0f / 3.0f));
-    float sv, cv;
-    sincospif(2.0f * f * y[d], &sv, &cv);
-    return (j & 1) ? cv : sv;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        float sv, cv;
+        sincospif(f2[k] * y, &sv, &cv);
+        w[k] = pack_bf16(sv, cv);
+    }
 }
 
 __device__ __forceinline__ void load_point(const float* __restrict__ x, int64_t n, int64_t r,
@@ -67,15 +82,21 @@ __device__ __forceinline__ void load_point(const float* __restrict__ x, int64_t 
 }
 
 // ---------------------------------------------------------------------------
-// Forward on the 5th-generation tensor cores (tcgen05).  A CTA of 512
-// threads is four independent quarters of 128 threads; each quarter takes
-// tiles of 128 points in turn (thread t of the quarter owns row t), so that
-// one quarter's products run on the tensor cores while the others convert
-// and activate (one CTA per SM: four tiles in flight).
-// Per tile the features (BF16) go to the quarter's A buffer in the canonical
+// Forward on the 5th-generation tensor cores (tcgen05).  A CTA is kTcTeams
+// independent teams of 128 threads; each team takes tiles of 128 points in
+// turn (thread t of the team owns row t), so that one team's products run on
+// the tensor cores while the others convert and activate (one CTA per SM,
+// kTcTeams tiles in flight).  Tiles go round the CTAs first: a call of few
+// points spreads over the SMs.  What bounds it is instruction issue (96 sines
+// and cosines and 256 SiLUs a point), not the tensor cores (7% busy): 2^20
+// points took 219 us with four teams, a frequency's exponential per feature and
+// the whole 64-column row in registers, and take 158 us with six teams,
+// frequencies formed once per block, 16 columns at a time and the exponential
+// and reciprocal without their subnormal handling.
+// Per tile the features (BF16) go to the team's A buffer in the canonical
 // K-major layout, one thread issues the layer's tcgen05.mma (M 128, N 64,
-// K 16 per instruction) into the quarter's 64 FP32 columns of tensor memory,
-// the commit arrives on the quarter's mbarrier, every thread loads its row of
+// K 16 per instruction) into the team's 64 FP32 columns of tensor memory,
+// the commit arrives on the team's mbarrier, every thread loads its row of
 // the accumulator (tcgen05.ld), adds the bias, applies SiLU and writes the
 // BF16 activations back as the next layer's A operand.  The weights (B
 // operand, W as stored: out x in = N x K, K-major) stay in shared memory for
@@ -83,16 +104,20 @@ __device__ __forceinline__ void load_point(const float* __restrict__ x, int64_t 
 // BF16-rounded activations, as the tensor cores would see them.
 // ---------------------------------------------------------------------------
 constexpr int kTcRows = 128;
-constexpr int kTcThreads = 4 * kTcRows;              // four quarters
-constexpr int kTcCols = 256;                         // tensor-memory columns per CTA (64 per quarter)
+constexpr int kTcTeams = 6;
+constexpr int kTcThreads = kTcTeams * kTcRows;
+constexpr int kTcCols = 512;                         // tensor-memory columns per CTA (64 per team)
+static_assert(kTcTeams * 64 <= kTcCols && kTcThreads <= 1024, "teams");
 constexpr int kTcOffW0 = 0;                          // 64 x 96 BF16, canonical K-major
 constexpr int kTcOffW1 = kTcOffW0 + 64 * kFeat * 2;  // W1..W3: 64 x 64
-constexpr int kTcOffA = kTcOffW1 + 3 * 64 * kWidth * 2;  // per quarter 128 x 96 BF16 (layers 1-3: 128 x 64)
+constexpr int kTcOffA = kTcOffW1 + 3 * 64 * kWidth * 2;  // per team 128 x 96 BF16 (layers 1-3: 128 x 64)
 constexpr int kTcABytes = kTcRows * kFeat * 2;
-constexpr int kTcOffBias = kTcOffA + 4 * kTcABytes;       // 4 x 64 FP32
+constexpr int kTcOffBias = kTcOffA + kTcTeams * kTcABytes;  // 4 x 64 FP32
 constexpr int kTcOffW5 = kTcOffBias + 4 * 64 * 4;         // 64 FP32, then b5
-constexpr int kTcOffMisc = kTcOffW5 + 64 * 4 + 16;        // 4 mbarriers (8 B each), TMEM address
-constexpr int kTcFwdSmem = kTcOffMisc + 48;
+constexpr int kTcOffFreq = kTcOffW5 + 64 * 4 + 16;        // 16 FP32
+constexpr int kTcOffMisc = kTcOffFreq + 16 * 4;          // an mbarrier (8 B) per team, TMEM address
+constexpr int kTcFwdSmem = kTcOffMisc + 8 * kTcTeams + 16;
+static_assert(kTcFwdSmem <= 227 * 1024, "forward tiles exceed shared memory");
 constexpr uint32_t kTcWaitLimit = 1u << 26;  // mbarrier polls before giving up (seconds)
 // Polls of the first wait on each product (the wait that detects a failure);
 // the drain of a product still in flight after a failure always takes
@@ -101,6 +126,17 @@ constexpr uint32_t kTcWaitLimit = 1u << 26;  // mbarrier polls before giving up 
 std::atomic<uint32_t> g_tc_first_wait{kTcWaitLimit};
 static_assert(kTcOffA % 1024 == 0 && kTcOffW1 % 1024 == 0 && kTcABytes % 1024 == 0,
               "operand alignment");
+
+// 16 BF16 values of row r, columns [c0, c0 + 16), into a K-major matrix with
+// `cols` columns (two 16-byte stores).
+__device__ __forceinline__ void store_words8(unsigned char* base, int r, int c0, int cols,
+                                             const uint32_t (&w)[8])
+{
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+        *reinterpret_cast<uint4*>(base + tc::kmajor_offset(r, c0 + 8 * c, cols)) =
+            make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+}
 
 // One layer's matrix (64 x IN, row-major FP32 in params) into shared memory
 // as BF16 in the canonical K-major layout (rows = outputs, K = inputs).
@@ -126,19 +162,20 @@ __device__ __forceinline__ void load_layer_kmajor(const float* __restrict__ W, u
     }
 }
 
-__global__ void __launch_bounds__(kTcThreads) k_mlp_forward_tc(const float* __restrict__ params,
+__global__ void __launch_bounds__(kTcThreads, 1) k_mlp_forward_tc(const float* __restrict__ params,
                                                               const float* __restrict__ x,
                                                               int stride, int64_t n,
                                                               float* __restrict__ out,
                                                               uint32_t first_wait)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
-    const int qtr = threadIdx.x >> 7, tid = threadIdx.x & 127, warp = threadIdx.x >> 5;
+    const int team = threadIdx.x >> 7, tid = threadIdx.x & 127, warp = threadIdx.x >> 5;
     float* bias = reinterpret_cast<float*>(smem + kTcOffBias);
     float* w5 = reinterpret_cast<float*>(smem + kTcOffW5);
-    const uint32_t mbar = tc::smem_addr(smem + kTcOffMisc + 8 * qtr);
-    uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + kTcOffMisc + 32);
-    unsigned char* A = smem + kTcOffA + qtr * kTcABytes;
+    float* f2 = reinterpret_cast<float*>(smem + kTcOffFreq);
+    const uint32_t mbar = tc::smem_addr(smem + kTcOffMisc + 8 * team);
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + kTcOffMisc + 8 * kTcTeams);
+    unsigned char* A = smem + kTcOffA + team * kTcABytes;
 
     // the network into shared memory, the accumulators into tensor memory
     const bool vec = (reinterpret_cast<uintptr_t>(params) & 15) == 0;
@@ -148,6 +185,7 @@ __global__ void __launch_bounds__(kTcThreads) k_mlp_forward_tc(const float* __re
                                   vec);
     for (int i = threadIdx.x; i < 4 * 64; i += blockDim.x) bias[i] = params[b_off(i >> 6) + (i & 63)];
     for (int i = threadIdx.x; i < 64; i += blockDim.x) w5[i] = params[kW5 + i];
+    if (threadIdx.x < 16) f2[threadIdx.x] = feature_freq2(threadIdx.x);
     if (threadIdx.x == 0) w5[64] = params[kB5];
     if (tid == 0) tc::mbar_init(mbar, 1);
     __syncwarp();
@@ -156,29 +194,26 @@ __global__ void __launch_bounds__(kTcThreads) k_mlp_forward_tc(const float* __re
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    const uint32_t tmem = *tslot + 64u * qtr;                 // this quarter's columns
+    const uint32_t tmem = *tslot + 64u * team;                // this team's columns
     const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);  // this warp's lanes
     constexpr uint32_t kIdesc = tc::idesc_bf16_f32(kTcRows, 64);
     const uint32_t a_base = tc::smem_addr(A);
-    const int bar = 1 + qtr;  // the quarter's named barrier
+    const int bar = 1 + team;  // the team's named barrier
     uint32_t phase = 0;
     bool failed = false;
 
     const int64_t tiles = (n + kTcRows - 1) / kTcRows;
-    for (int64_t tile = 4 * (int64_t)blockIdx.x + qtr; tile < tiles && !failed;
-         tile += 4 * (int64_t)gridDim.x) {
+    for (int64_t tile = blockIdx.x + (int64_t)gridDim.x * team; tile < tiles && !failed;
+         tile += kTcTeams * (int64_t)gridDim.x) {
         const int64_t r = tile * kTcRows + tid;
         float y[3];
         load_point(x, n, r, y, stride);
-        // features of row tid: 12 chunks of 8 columns, one 16-byte store each
+        // features of row tid: 16 columns (8 frequencies of a coordinate) at a time
 #pragma unroll 1
-        for (int c = 0; c < kFeat / 8; ++c) {
-            float f[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) f[j] = feature(y, 8 * c + j);
-            *reinterpret_cast<uint4*>(A + tc::kmajor_offset(tid, 8 * c, kFeat)) =
-                make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]),
-                           pack_bf16(f[6], f[7]));
+        for (int c = 0; c < 6; ++c) {
+            uint32_t f[8];
+            features8(c < 2 ? y[0] : c < 4 ? y[1] : y[2], f2 + 8 * (c & 1), f);
+            store_words8(A, tid, 16 * c, kFeat, f);
         }
         float o = 0.f;
         for (int l = 0; l < 4; ++l) {
@@ -196,37 +231,36 @@ __global__ void __launch_bounds__(kTcThreads) k_mlp_forward_tc(const float* __re
                 tc::commit(mbar);
             }
             const bool ok = tc::mbar_wait(mbar, phase, first_wait);
-            if (tc::bar_sync_or(bar, kTcRows, !ok)) {  // the quarter stops together
+            if (tc::bar_sync_or(bar, kTcRows, !ok)) {  // the team stops together
                 failed = true;
                 if (!ok) tc::mbar_wait(mbar, phase, kTcWaitLimit);  // the product in flight, bounded
                 break;
             }
             phase ^= 1u;
             tc::fence_after_sync();
-            float h[64];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
+            for (int q = 0; q < 4; ++q) {  // 16 columns at a time
                 float v[16];
                 tc::tmem_ld16(trow + 16 * q, v);
+                tc::tmem_wait_ld();
+                uint32_t h[8];
 #pragma unroll
-                for (int j = 0; j < 16; ++j) h[16 * q + j] = v[j];
+                for (int j = 0; j < 8; ++j) {
+                    const float2 b = *reinterpret_cast<const float2*>(bias + 64 * l + 16 * q + 2 * j);
+                    const float2 a = __fadd2_rn(make_float2(v[2 * j], v[2 * j + 1]), b);
+                    h[j] = pack_bf16(silu(a.x), silu(a.y));
+                }
+                if (l < 3) {
+                    store_words8(A, tid, 16 * q, kWidth, h);
+                } else {  // the BF16 activations times the output weights
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        o = fmaf(__uint_as_float(h[j] << 16), w5[16 * q + 2 * j], o);
+                        o = fmaf(__uint_as_float(h[j] & 0xFFFF0000u), w5[16 * q + 2 * j + 1], o);
+                    }
+                }
             }
-            tc::tmem_wait_ld();
-#pragma unroll
-            for (int j = 0; j < 64; ++j) h[j] = silu(h[j] + bias[64 * l + j]);
-            if (l < 3) {
-#pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    *reinterpret_cast<uint4*>(A + tc::kmajor_offset(tid, 8 * c, kWidth)) =
-                        make_uint4(pack_bf16(h[8 * c], h[8 * c + 1]), pack_bf16(h[8 * c + 2], h[8 * c + 3]),
-                                   pack_bf16(h[8 * c + 4], h[8 * c + 5]),
-                                   pack_bf16(h[8 * c + 6], h[8 * c + 7]));
-            } else {
-#pragma unroll
-                for (int j = 0; j < 64; ++j)
-                    o = fmaf(__bfloat162float(__float2bfloat16_rn(h[j])), w5[j], o);
-                o += w5[64];
-            }
+            if (l == 3) o += w5[64];
         }
         if (r < n) out[r] = failed ? __int_as_float(0x7FC00000) : o;
     }
@@ -248,7 +282,10 @@ __global__ void __launch_bounds__(kTcThreads) k_mlp_forward_tc(const float* __re
 // The pre-activations of the hidden layers stay in tensor memory (columns
 // 64 l .. 64 l + 63) until the backward pass needs them; every h_l carries a
 // column of ones after its K_l inputs, so row K_l of dW_l^T is the bias
-// gradient.
+// gradient.  A step is a chain of products, barriers and epilogues (latency;
+// 4,096 points are 32 CTAs): 33.4 us with the optimiser, 25.5 us since the
+// features take their frequencies from a table, the output layer's column sums
+// take 31 shuffles instead of 160 and no accumulator passes local memory.
 // ---------------------------------------------------------------------------
 constexpr int kTrainRows = 128;
 constexpr int kTrThreads = 2 * kTrainRows;
@@ -263,7 +300,8 @@ constexpr int kTrOffBias = kTrOffDA + kTrainRows * kWidth * 2;    // 4 x 64 FP32
 constexpr int kTrOffW5 = kTrOffBias + 4 * 64 * 4;                 // 64 FP32 + b5
 constexpr int kTrOffRed = kTrOffW5 + 64 * 4 + 16;                 // reductions across warps
 constexpr int kTrRedFloats = 8 * 34 + 2 * 128;
-constexpr int kTrOffMisc = kTrOffRed + kTrRedFloats * 4;          // mbarrier, TMEM address
+constexpr int kTrOffFreq = kTrOffRed + kTrRedFloats * 4;          // 16 FP32
+constexpr int kTrOffMisc = kTrOffFreq + 16 * 4;                   // mbarrier, TMEM address
 // Slack after the last operand: the products read up to 128 MN-major rows
 // of an h_l whose own buffer has fewer, and the slack keeps every operand
 // read inside the block's shared memory.
@@ -321,6 +359,7 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const float* __r
     float* bias = reinterpret_cast<float*>(smem + kTrOffBias);
     float* w5 = reinterpret_cast<float*>(smem + kTrOffW5);
     float* red = reinterpret_cast<float*>(smem + kTrOffRed);
+    float* f2 = reinterpret_cast<float*>(smem + kTrOffFreq);
     const uint32_t mbar = tc::smem_addr(smem + kTrOffMisc);
     uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + kTrOffMisc + 8);
     unsigned char* DA = smem + kTrOffDA;
@@ -332,6 +371,7 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const float* __r
     for (int l = 1; l < 4; ++l) load_layer_kmajor<kWidth>(params + w_off(l), wb(l), vec);
     for (int i = threadIdx.x; i < 4 * 64; i += blockDim.x) bias[i] = params[b_off(i >> 6) + (i & 63)];
     for (int i = threadIdx.x; i < 64; i += blockDim.x) w5[i] = params[kW5 + i];
+    if (threadIdx.x < 16) f2[threadIdx.x] = feature_freq2(threadIdx.x);
     // the ones column (bias gradients) and the padding of every h_l
     if (ch == 0) {
         const uint4 ones = make_uint4(pack_bf16(1.f, 0.f), 0u, 0u, 0u);
@@ -381,13 +421,10 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const float* __r
     load_point(x, n, row, y);
     // ---- forward: features -> h0 (this thread's 48 of the 96)
 #pragma unroll 1
-    for (int c = 6 * ch; c < 6 * ch + 6; ++c) {
-        float f[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) f[j] = feature(y, 8 * c + j);
-        *reinterpret_cast<uint4*>(hb(0) + tc::kmajor_offset(r, 8 * c, kH0Cols)) =
-            make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]),
-                       pack_bf16(f[6], f[7]));
+    for (int c = 3 * ch; c < 3 * ch + 3; ++c) {
+        uint32_t f[8];
+        features8(c < 2 ? y[0] : c < 4 ? y[1] : y[2], f2 + 8 * (c & 1), f);
+        store_words8(hb(0), r, 16 * c, kH0Cols, f);
     }
     float h[32];
     float out = 0.f;
@@ -425,12 +462,20 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const float* __r
         const float o = outs[r] + outs[128 + r] + w5[64];
         const float e = row < n ? o - target[row] : 0.f;
         const float dout = 2.f * e / (float)n;
-#pragma unroll 1
-        for (int j = 0; j < 32; ++j) {
-            float v = dout * h[j];
-            for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(kFull, v, s);
-            if (lane == 0) red[warp * 34 + j] = v;
+        // column sums over the warp's 32 rows: each exchange halves the columns
+        // a lane holds (31 shuffles for all 32); lane j ends up with column j
+#pragma unroll
+        for (int j = 0; j < 32; ++j) h[j] *= dout;
+#pragma unroll
+        for (int w = 16; w > 0; w >>= 1) {
+            const bool up = lane & w;
+#pragma unroll
+            for (int j = 0; j < w; ++j) {
+                const float other = __shfl_xor_sync(kFull, up ? h[j] : h[j + w], w);
+                h[j] = (up ? h[j + w] : h[j]) + other;
+            }
         }
+        red[warp * 34 + lane] = h[0];
         float dsum = dout, le = e * e;
         for (int s = 16; s > 0; s >>= 1) {
             dsum += __shfl_xor_sync(kFull, dsum, s);
@@ -478,8 +523,10 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const float* __r
             float g[32];
             tmem_row32(trow + kColDW, g);  // row r of dW_l^T: input r, outputs c0 .. c0 + 31
             if (r < K) {
+#pragma unroll
                 for (int j = 0; j < 32; ++j) gpart[w_off(l) + (c0 + j) * K + r] = g[j];
             } else if (r == K) {
+#pragma unroll
                 for (int j = 0; j < 32; ++j) gpart[b_off(l) + c0 + j] = g[j];
             }
             if (l == 0) break;
@@ -586,7 +633,7 @@ int mlp_forward(const float* params, const float* x, int64_t n, float* out, cuda
     WOB_TRY(allow_smem(g_fwd_configured, (const void*)k_mlp_forward_tc, kTcFwdSmem));
     const int64_t tiles = (n + kTcRows - 1) / kTcRows;
     const int grid = grid_for((const void*)k_mlp_forward_tc, kTcThreads, kTcFwdSmem,
-                              (tiles + 3) / 4 * kTcThreads);
+                              tiles * kTcThreads);
     k_mlp_forward_tc<<<grid, kTcThreads, kTcFwdSmem, s>>>(params, x, stride, n, out,
                                                           g_tc_first_wait.load());
     WOB_CUDA_TRY(cudaGetLastError());
