@@ -130,7 +130,6 @@ void fill_params(WalkParams& p, const wob_problem* prob, const float* queries,
     p.iter_limit = prob->iter_limit > 0 ? prob->iter_limit : (int)(4 * b.n_wide + 64);
     p.stack_levels = b.wide_levels;
     p.verts = m.verts;
-    p.verts_d = m.verts_d;
     p.tris = m.tris;
     p.tri_n = m.tri_n;
     p.tri_f = m.tri_f;

@@ -1,7 +1,7 @@
 // walk.cu -- the walk-on-boundary kernels:
 //   k_dl_lines   Dirichlet problems, double-layer formulation, ray (line)
 //                sampling with all-hits queries (Sec. 4.1, 4.4.1)
-//   k_sl_walks_ff / k_sl_walks
+//   k_sl_walks_ff / k_sl_walks_ris
 //                Neumann / Robin problems, single-layer formulation, area
 //                sampling / resampled importance sampling (Sec. 4.3)
 //   k_nd_lines   Neumann problems through the direct boundary integral
@@ -52,6 +52,10 @@ constexpr int64_t kGroupWalksPerSm = 200;
 #ifndef WOB_SL_MIN_BLOCKS
 #define WOB_SL_MIN_BLOCKS 6
 #endif
+// Resampled single-layer walks: 7 blocks of 128 threads per SM (72 registers).  On
+// 1.05e6 walks of the mixed torus 6 blocks took 1.61 ms, 7 1.52, 8 (64 registers)
+// 1.54.
+constexpr int kRisBlocks = 7;
 
 // Tiles of 32 consecutive walks of one problem from its global counter
 // (dynamic balance), the 64-bit bookkeeping of the two tiles under way and
@@ -300,176 +304,6 @@ __device__ __forceinline__ int64_t area_pick(const WalkParams& p, uint32_t hi, u
     return a;
 }
 
-// Area-uniform boundary point of stream (q, w, step, attempt): triangle j (original
-// order) by inverse CDF of the areas (area_pick), then a uniform point on it
-// (square-root warp), barycentrics b0..b2; n = the triangle's unit normal.
-struct AreaPoint {
-    int64_t j;
-    double3 y, n;
-    double b0, b1, b2;
-};
-
-__device__ __forceinline__ AreaPoint area_point(const WalkParams& p, StreamKey key, uint32_t q,
-                                                uint32_t w, uint32_t step, uint32_t attempt = 0u)
-{
-    AreaPoint a;
-    const u32x4 u = stream_block(key, q, w, step, kPurposeArea, attempt, 0u);
-    const int64_t lo = area_pick(p, u.x, u.y);
-    const double su = sqrt(u24(u.z)), u2 = u24(u.w);
-    a.b0 = 1.0 - su;
-    a.b1 = su * (1.0 - u2);
-    a.b2 = su * u2;
-    const int32_t* t = p.tris + 3 * lo;
-    const double* v0 = p.verts_d + 3 * (int64_t)__ldg(t);
-    const double* v1 = p.verts_d + 3 * (int64_t)__ldg(t + 1);
-    const double* v2 = p.verts_d + 3 * (int64_t)__ldg(t + 2);
-    a.y = make_double3(a.b0 * __ldg(v0) + a.b1 * __ldg(v1) + a.b2 * __ldg(v2),
-                       a.b0 * __ldg(v0 + 1) + a.b1 * __ldg(v1 + 1) + a.b2 * __ldg(v2 + 1),
-                       a.b0 * __ldg(v0 + 2) + a.b1 * __ldg(v1 + 2) + a.b2 * __ldg(v2 + 2));
-    const double2 nxy = __ldg(reinterpret_cast<const double2*>(p.tri_n + lo));
-    const double nz = __ldg(reinterpret_cast<const double*>(p.tri_n + lo) + 2);
-    a.n = make_double3(nxy.x, nxy.y, nz);
-    a.j = lo;
-    return a;
-}
-
-// Transition kernel of the single-layer recursion from x (condition bx,
-// normal nx; bx < 0: the query) to y, without the 1/p of the sampling
-// (Table 1; Sec. 4.3 for the Dirichlet parts of mixed problems): G (query),
-// -2 phi dG/dn_x (Neumann), -2 phi (dG/dn_x + alpha G) (Robin), -(k/p_k) G
-// (Dirichlet, moving branch); dG/dn_x = (y - x) . n_x / (4 pi r^3).  0 for
-// r < rmin.
-__device__ __forceinline__ double sl_kernel(const WalkParams& p, int bx, double3 x, double3 nx,
-                                            double3 y, double rmin)
-{
-    const double rx = y.x - x.x, ry = y.y - x.y, rz = y.z - x.z;
-    const double rl = sqrt(rx * rx + ry * ry + rz * rz);
-    if (rl < rmin) return 0.0;
-    const double G = 1.0 / (kFourPi * rl);
-    if (bx < 0) return G;
-    if (bx == WOB_BC_DIRICHLET) return -((double)p.kmix / (double)p.pk) * G;
-    const double dgdn = (rx * nx.x + ry * nx.y + rz * nx.z) / (kFourPi * rl * rl * rl);
-    const double phi = (double)p.phi;
-    if (bx == WOB_BC_NEUMANN) return -2.0 * phi * dgdn;
-    return -2.0 * phi * (dgdn + (double)p.alpha * G);
-}
-
-// sl_data with the point-source field in FP32 from an FP64 difference and
-// the normal derivative n . grad h in FP64 (it cancels where the field runs
-// along the surface); polynomial and P1 data as sl_data (a polynomial's
-// monomials cancel, and its FP64 evaluation costs little).
-__device__ __forceinline__ double sl_data32(const WalkParams& p, int64_t j, double3 y, double b0,
-                                            double b1, double b2, double3 n, int bc)
-{
-    const DataDev& D = p.data;
-    if (D.mode == WOB_DATA_VERTEX_P1) {
-        const int32_t* t = D.tris + 3 * j;
-        return b0 * __ldg(D.vdata + t[0]) + b1 * __ldg(D.vdata + t[1]) + b2 * __ldg(D.vdata + t[2]);
-    }
-    if (D.mode == WOB_DATA_POLY) return sl_data(p, j, y, b0, b1, b2, n, bc);
-    const double dx = y.x - D.x0[0], dy = y.y - D.x0[1], dz = y.z - D.x0[2];
-    const float ri = rsqrtf((float)(dx * dx + dy * dy + dz * dz));
-    const float h = D.scale * ri;
-    const float f = -h * ri * ri;
-    const float gx = f * (float)dx, gy = f * (float)dy, gz = f * (float)dz;
-    if (bc == WOB_BC_DIRICHLET) return (double)h;
-    const double dhdn = n.x * (double)gx + n.y * (double)gy + n.z * (double)gz;
-    return bc == WOB_BC_ROBIN ? dhdn + (double)p.alpha * (double)h : dhdn;
-}
-
-// Single-layer walks (Table 1, Sec. 4.3), one thread per walk:
-// u(x0) = int G mu and mu(x) = int K(x, y) mu(y) + src(x), src = 2 phi q
-// (Neumann), 2 phi (q + alpha h) (Robin), k u_D (Dirichlet parts of mixed
-// problems, whose mu(x) = mu(x) - k S mu + k u_D is sampled by moving with
-// probability p_k or staying at x with weight 1 / (1 - p_k)).  The last
-// source is halved (Sec. 4.1.2).  This kernel (FP64 kernels) serves
-// resampled importance sampling (Talbot et al. 2005): the next point is
-// drawn from p.ris area-uniform candidates with target |K|, weight sign(K)
-// |Gamma| (sum of |K| over the candidates) / ris.  Plain area sampling runs
-// in k_sl_walks_ff.
-template <bool DEBUG>
-__global__ void __launch_bounds__(128) k_sl_walks(WalkParams p)
-{
-    const StreamKey key{p.key0, p.key1};
-    const int64_t total = p.Q * (int64_t)p.N;
-    const double phi = (double)p.phi;
-    const double area = p.area;
-    const double rmin = 1e-12 * p.L;
-    const int uniform_bc = p.kind == WOB_ROBIN_SL ? WOB_BC_ROBIN : WOB_BC_NEUMANN;
-    double wc[kMaxRis];
-    const int lane = threadIdx.x & 31;
-    // warp-uniform loop over groups of 32 consecutive walks
-    for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); base < total;
-         base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t idx = base + lane;
-        const bool live = idx < total;
-        const int64_t qi = live ? idx / p.N : 0;
-        const int64_t wi = idx - qi * p.N;
-        double value = 0.0;
-        if (live) {
-            const uint32_t q = p.q_base + (uint32_t)qi;
-            const uint32_t w = (uint32_t)(p.walk_begin + wi);
-            double3 x = make_double3(p.queries[3 * qi], p.queries[3 * qi + 1], p.queries[3 * qi + 2]);
-            double3 nx = make_double3(0.0, 0.0, 0.0);
-            int bx = -1;
-            int64_t jx = -1;
-            double S = 0.0, P = 1.0, W0 = 0.0;
-            for (int k = 0; k < p.M; ++k) {
-                bool stay = false;
-                if (bx == WOB_BC_DIRICHLET) {
-                    const u32x4 u = stream_block(key, q, w, (uint32_t)k, kPurposeBranch, 0u, 0u);
-                    stay = u24(u.x) >= (double)p.pk;
-                }
-                AreaPoint a;
-                double wfac;
-                if (stay) {
-                    a.j = jx;
-                    a.y = x;
-                    a.n = nx;
-                    a.b0 = a.b1 = a.b2 = 0.0;  // mixed problems take analytic data
-                    wfac = 1.0 / (1.0 - (double)p.pk);
-                } else {
-                    double sumw = 0.0;
-                    for (int c = 0; c < p.ris; ++c) {
-                        const AreaPoint ac = area_point(p, key, q, w, (uint32_t)k, (uint32_t)c);
-                        wc[c] = fabs(sl_kernel(p, bx, x, nx, ac.y, rmin));
-                        sumw += wc[c];
-                    }
-                    if (!(sumw > 0.0)) break;  // every candidate has a zero kernel
-                    const u32x4 u = stream_block(key, q, w, (uint32_t)k, kPurposeRis, 0u, 0u);
-                    const double target = u53(u.x, u.y) * sumw;
-                    double acc = 0.0;
-                    int pick = p.ris - 1;
-                    for (int c = 0; c < p.ris; ++c) {
-                        acc += wc[c];
-                        if (acc > target) {
-                            pick = c;
-                            break;
-                        }
-                    }
-                    a = area_point(p, key, q, w, (uint32_t)k, (uint32_t)pick);
-                    const double K = sl_kernel(p, bx, x, nx, a.y, rmin);
-                    wfac = (K > 0.0 ? 1.0 : -1.0) * area * sumw / (double)p.ris;
-                }
-                if (k == 0) W0 = wfac; else P *= wfac;
-                const int by = p.bc_type ? (int)__ldg(p.bc_type + a.j) : uniform_bc;
-                const double dat = sl_data32(p, a.j, a.y, a.b0, a.b1, a.b2, a.n, by);
-                double src = by == WOB_BC_DIRICHLET ? (double)p.kmix * dat : 2.0 * phi * dat;
-                if (k == p.M - 1) src *= 0.5;
-                S = fma(P, src, S);
-                x = a.y;
-                nx = a.n;
-                bx = by;
-                jx = a.j;
-            }
-            value = W0 * S;
-            if (p.per_walk) p.per_walk[idx] = value;
-            if (DEBUG && p.walk_flag) p.walk_flag[idx] = 0;
-        }
-        if (p.part) add_tile_partials(value, live, qi, wi, p.tpq, p.part);
-    }
-}
-
 // ---------------------------------------------------------------------------
 // Single-layer walks with area sampling in compensated FP32.  Each sample
 // point is kept as its triangle's first vertex v0 (FP32, exact) plus the
@@ -580,9 +414,15 @@ __device__ __forceinline__ float sl_data_ff(const WalkParams& p, int64_t j, cons
     return bc == WOB_BC_ROBIN ? __fmaf_rn(p.alpha, h, dhdn) : dhdn;
 }
 
-// The single-layer walks of k_sl_walks for area sampling (p.ris <= 1), in
-// the compensated FP32 arithmetic above; the transition kernel and the
-// sources are those of sl_kernel / sl_data (Table 1, Sec. 4.3).
+// Single-layer walks (Table 1, Sec. 4.3) with area sampling (p.ris <= 1), one
+// thread per walk, in the compensated FP32 arithmetic above:
+// u(x0) = int G mu and mu(x) = int K(x, y) mu(y) + src(x) with K = G (query),
+// -2 phi dG/dn_x (Neumann), -2 phi (dG/dn_x + alpha G) (Robin), -(k/p_k) G
+// (Dirichlet, moving branch), dG/dn_x = (y - x) . n_x / (4 pi r^3), 0 for
+// r < 1e-12 L; src = 2 phi q (Neumann), 2 phi (q + alpha h) (Robin), k u_D
+// (Dirichlet parts of mixed problems, whose mu(x) = mu(x) - k S mu + k u_D is
+// sampled by moving with probability p_k or staying at x with weight
+// 1 / (1 - p_k)).  The last source is halved (Sec. 4.1.2).
 template <bool DEBUG>
 __global__ void __launch_bounds__(128, WOB_SL_MIN_BLOCKS) k_sl_walks_ff(WalkParams p)
 {
@@ -685,6 +525,230 @@ __global__ void __launch_bounds__(128, WOB_SL_MIN_BLOCKS) k_sl_walks_ff(WalkPara
                 jx = j;
             }
             value = (double)W0 * S;
+            if (p.per_walk) p.per_walk[idx] = value;
+            if (DEBUG && p.walk_flag) p.walk_flag[idx] = 0;
+        }
+        if (p.part) add_tile_partials(value, live, qi, wi, p.tpq, p.part);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Single-layer walks with resampled importance sampling (Talbot et al. 2005):
+// the next point is drawn from p.ris area-uniform candidates with target |K|,
+// weight sign(K) |Gamma| (sum of |K| over the candidates) / ris; walks, K and
+// sources as in k_sl_walks_ff.  The pick compares running sums of |K|, so a
+// rounding can move it to another candidate: points, kernels and sums are
+// float-float (44 bits and more; a pick moves about once in 10^11 draws), and
+// the walk's weights, terms and sums FP64.  What bounds it is issue: some 400
+// FP32 instructions a candidate, where about 60 FP64 instructions, each worth
+// 64 FP32 issue slots on this GPU, took 14.1 ms for 1.05e6 walks x 4 vertices x 16
+// candidates (200,000 triangles).  Now 1.52 ms; 2.5 ms while lanes that stayed
+// or had another condition branched apart (16 of 32 active).
+// ---------------------------------------------------------------------------
+
+// 1 / sqrt(a) for a normal a: the fast root y, corrected to second order in
+// e = 1 - a y^2 (y (1 + e / 2 + 3 e^2 / 8); e ~ 1e-7).
+__device__ __forceinline__ ff ff_rsqrt(ff a)
+{
+    const float y = rsqrt_ftz(a.hi);
+    const ff t = ff_mul(a, two_prod(y, y));
+    const float e = rn_sub(rn_sub(1.f, t.hi), t.lo);
+    return fast_two_sum(y, rn_mul(rn_mul(y, e), rn_fma(0.375f, e, 0.5f)));
+}
+
+// K without its constant factor, at the candidate y of the vertex x (condition
+// bx, bx < 0: the query), as float-float and in units of 2^s_e lengths (scale =
+// 2^-s_e, about 1 / L, and alpha in these units: the powers of r stay in FP32's
+// range on boundaries of any size): 1 / r (query, Dirichlet), r . n_x / r^3
+// (Neumann), (r . n_x + alpha r^2) / r^3 (Robin).  Candidates closer than about L / 128 are left
+// to ris_kernel_close: their K, the largest of all and cancelling the most (r . n_x
+// falls as r^2), dominate the variance, and stay what FP64 gives for them.
+constexpr float kRisClose2 = 0x1p-14f;
+
+__device__ __forceinline__ ff ris_kernel(int bx, const FFPoint& x, const FFPoint& y, float scale,
+                                         float alpha, bool& close)
+{
+    ff r[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        r[c] = ff_add(two_sum(y.v0[c], -x.v0[c]), ff_sub(y.p[c], x.p[c]));
+        r[c] = {rn_mul(r[c].hi, scale), rn_mul(r[c].lo, scale)};
+    }
+    const ff rr = ff_dot3(r, r);
+    close = rr.hi < kRisClose2;
+    // every condition's lanes together: alpha is 0 but on Robin parts
+    const ff ri = ff_rsqrt(rr);
+    const ff num = ff_add(ff_dot3(x.n, r), ff_mul_f(rr, bx == WOB_BC_ROBIN ? alpha : 0.f));
+    const ff K = ff_mul(ff_mul(num, ri), ff_mul(ri, ri));
+    return bx < 0 || bx == WOB_BC_DIRICHLET ? ri : K;
+}
+
+// The same value for a candidate within L / 128 of the vertex, all in FP64 and
+// absolute coordinates; triangle jx and the uniforms ux (jx < 0: the query xq),
+// jy and uy.  Rare (one candidate in 10^4 on a torus), and out of line.
+__device__ __noinline__ ff ris_kernel_close(const WalkParams& p, int bx, int64_t jx, float2 ux,
+                                            const float* xq, int64_t jy, float2 uy, float scale)
+{
+    auto point = [&](int64_t j, float2 u) {
+        const double su = sqrt((double)u.x), u2 = (double)u.y;
+        const double b0 = 1.0 - su, b1 = su * (1.0 - u2), b2 = su * u2;
+        const int32_t* t = p.tris + 3 * j;
+        const float *v0 = p.verts + 3 * (int64_t)t[0], *v1 = p.verts + 3 * (int64_t)t[1],
+                    *v2 = p.verts + 3 * (int64_t)t[2];
+        return make_double3(b0 * (double)v0[0] + b1 * (double)v1[0] + b2 * (double)v2[0],
+                            b0 * (double)v0[1] + b1 * (double)v1[1] + b2 * (double)v2[1],
+                            b0 * (double)v0[2] + b1 * (double)v1[2] + b2 * (double)v2[2]);
+    };
+    const double3 x = jx < 0 ? make_double3(xq[0], xq[1], xq[2]) : point(jx, ux), y = point(jy, uy);
+    const double rx = y.x - x.x, ry = y.y - x.y, rz = y.z - x.z;
+    const double r2 = rx * rx + ry * ry + rz * rz, rl = sqrt(r2);
+    if (rl < 1e-12 * p.L) return {0.f, 0.f};
+    if (bx < 0 || bx == WOB_BC_DIRICHLET) return ff_split(1.0 / (rl * (double)scale));
+    const NormalArea n = p.tri_n[jx];
+    double num = rx * n.nx + ry * n.ny + rz * n.nz;
+    if (bx == WOB_BC_ROBIN) num += (double)p.alpha * r2;
+    return ff_split(num / (r2 * rl * (double)scale * (double)scale));
+}
+
+// sl_data at y (uniforms su_u, u2 of its draw) with the point-source field in
+// FP32 from a float-float difference and the normal derivative n . grad h in
+// FP64 (it cancels where the field runs along the surface).
+__device__ __forceinline__ double ris_data(const WalkParams& p, int64_t j, const FFPoint& y,
+                                           float su_u, float u2, int bc)
+{
+    const DataDev& D = p.data;
+    if (D.mode != WOB_DATA_POINT) {
+        const double su = ff_join(ff_sqrt(su_u));
+        double3 yd, nd;
+        yd.x = (double)y.v0[0] + ff_join(y.p[0]);
+        yd.y = (double)y.v0[1] + ff_join(y.p[1]);
+        yd.z = (double)y.v0[2] + ff_join(y.p[2]);
+        nd = make_double3(ff_join(y.n[0]), ff_join(y.n[1]), ff_join(y.n[2]));
+        return sl_data(p, j, yd, 1.0 - su, su * (1.0 - (double)u2), su * (double)u2, nd, bc);
+    }
+    ff d[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) d[c] = ff_add(two_sum(y.v0[c], -D.x0[c]), y.p[c]);
+    const float ri = rsqrtf(ff_dot3(d, d).hi);
+    const float h = D.scale * ri;
+    if (bc == WOB_BC_DIRICHLET) return (double)h;
+    const float f = -h * ri * ri;
+    double dhdn = 0.0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) dhdn = fma(ff_join(y.n[c]), (double)(f * d[c].hi), dhdn);
+    return bc == WOB_BC_ROBIN ? dhdn + (double)p.alpha * (double)h : dhdn;
+}
+
+template <bool DEBUG>
+__global__ void __launch_bounds__(128, kRisBlocks) k_sl_walks_ris(WalkParams p)
+{
+    const StreamKey key{p.key0, p.key1};
+    const int64_t total = p.Q * (int64_t)p.N;
+    const double phi = (double)p.phi;
+    const int se = ilogb(p.L);
+    const float scale = scalbnf(1.f, -se), alpha = p.alpha / scale;
+    // |Gamma| / ris times the constant factors of K and the units' powers
+    const double wq = p.area / (double)p.ris / kFourPi * (double)scale;       // G
+    const double wd = wq * ((double)p.kmix / (double)p.pk);                   // (k / p_k) G
+    const double wl = 2.0 * wq * (double)scale;                               // 2 dG/dn_x
+    const int uniform_bc = p.kind == WOB_ROBIN_SL ? WOB_BC_ROBIN : WOB_BC_NEUMANN;
+    ff wc[kMaxRis];
+    const int lane = threadIdx.x & 31;
+    // warp-uniform loop over groups of 32 consecutive walks
+    for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); base < total;
+         base += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t idx = base + lane;
+        const bool live = idx < total;
+        const int64_t qi = live ? idx / p.N : 0;
+        const int64_t wi = live ? idx - qi * p.N : 0;
+        const uint32_t q = p.q_base + (uint32_t)qi;
+        const uint32_t w = (uint32_t)(p.walk_begin + wi);
+        FFPoint x;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            x.v0[c] = p.queries[3 * qi + c];
+            x.p[c] = {0.f, 0.f};
+            x.n[c] = {0.f, 0.f};
+        }
+        int bx = -1;
+        int64_t jx = -1;
+        float ux = 0.f, u2x = 0.f;
+        double S = 0.0, P = 1.0, W0 = 0.0;
+        bool going = live;
+        // every lane takes part in every step: a walk that stays, or has ended,
+        // draws its candidates too and drops them (the warp would wait for the
+        // others' all the same)
+        for (int k = 0; k < p.M && __any_sync(kAllLanes, going); ++k) {
+            bool stay = false;
+            if (bx == WOB_BC_DIRICHLET) {
+                const u32x4 u = stream_block(key, q, w, (uint32_t)k, kPurposeBranch, 0u, 0u);
+                stay = u24f(u.x) >= p.pk;  // both exact in FP32
+            }
+            FFPoint y;
+            ff sumw = {0.f, 0.f};
+            float b0, b1, b2;
+            for (int c = 0; c < p.ris; ++c) {
+                __syncwarp();
+                const u32x4 u = stream_block(key, q, w, (uint32_t)k, kPurposeArea, (uint32_t)c, 0u);
+                const int64_t j = area_pick(p, u.x, u.y);
+                __syncwarp();  // the searches differ in length
+                frame_point_ff(p, j, u.z, u.w, y, b0, b1, b2);
+                bool close;
+                ff K = ris_kernel(bx, x, y, scale, alpha, close);
+                if (close && going && !stay)
+                    K = ris_kernel_close(p, bx, jx, make_float2(ux, u2x), p.queries + 3 * qi, j,
+                                         make_float2(u24f(u.z), u24f(u.w)), scale);
+                wc[c] = K;
+                sumw = ff_add(sumw, K.hi < 0.f ? ff{-K.hi, -K.lo} : K);
+            }
+            __syncwarp();
+            if (!stay && !(sumw.hi > 0.f)) going = false;  // every candidate has a zero kernel
+            if (going) {
+                double wfac;
+                if (stay) {
+                    wfac = 1.0 / (1.0 - (double)p.pk);
+                } else {
+                    u32x4 u = stream_block(key, q, w, (uint32_t)k, kPurposeRis, 0u, 0u);
+                    // the 53-bit uniform as 24 + 29 bits
+                    const ff t = ff_mul(fast_two_sum(rn_mul((float)(u.x >> 8), 0x1p-24f),
+                                                     rn_mul((float)(((u.x & 0xFFu) << 21) | (u.y >> 11)),
+                                                            0x1p-53f)),
+                                        sumw);
+                    ff acc = {0.f, 0.f};
+                    int pick = p.ris - 1;
+                    for (int c = 0; c < p.ris; ++c) {
+                        const ff K = wc[c];
+                        acc = ff_add(acc, K.hi < 0.f ? ff{-K.hi, -K.lo} : K);
+                        if (acc.hi > t.hi || (acc.hi == t.hi && acc.lo > t.lo)) {
+                            pick = c;
+                            break;
+                        }
+                    }
+                    u = stream_block(key, q, w, (uint32_t)k, kPurposeArea, (uint32_t)pick, 0u);
+                    const int64_t j = area_pick(p, u.x, u.y);
+                    frame_point_ff(p, j, u.z, u.w, y, b0, b1, b2);
+                    // sign(K): positive for G, -phi sign(wc) on Neumann and Robin
+                    // parts, negative on Dirichlet parts (and for a zero kernel)
+                    const float sg = bx < 0 ? wc[pick].hi : bx == WOB_BC_DIRICHLET ? -1.f
+                                                          : -(float)p.phi * wc[pick].hi;
+                    const double wk = bx < 0 ? wq : bx == WOB_BC_DIRICHLET ? wd : wl;
+                    wfac = (sg > 0.f ? wk : -wk) * ff_join(sumw);
+                    x = y;
+                    jx = j;
+                    ux = u24f(u.z);
+                    u2x = u24f(u.w);
+                }
+                if (k == 0) W0 = wfac; else P *= wfac;
+                const int by = p.bc_type ? (int)__ldg(p.bc_type + jx) : uniform_bc;
+                const double dat = ris_data(p, jx, x, ux, u2x, by);
+                double src = by == WOB_BC_DIRICHLET ? (double)p.kmix * dat : 2.0 * phi * dat;
+                if (k == p.M - 1) src *= 0.5;
+                S = fma(P, src, S);
+                bx = by;
+            }
+        }
+        const double value = W0 * S;
+        if (live) {
             if (p.per_walk) p.per_walk[idx] = value;
             if (DEBUG && p.walk_flag) p.walk_flag[idx] = 0;
         }
@@ -1374,11 +1438,11 @@ int launch_sl_walks(const WalkParams& p, bool debug, cudaStream_t s)
 {
     const int threads = 128;
     const int64_t work = p.Q * (int64_t)p.N;
-    if (p.ris > 1) {  // resampling: FP64 kernels (its pick compares running sums)
+    if (p.ris > 1) {
         if (debug)
-            k_sl_walks<true><<<grid_for((const void*)k_sl_walks<true>, threads, 0, work), threads, 0, s>>>(p);
+            k_sl_walks_ris<true><<<grid_for((const void*)k_sl_walks_ris<true>, threads, 0, work), threads, 0, s>>>(p);
         else
-            k_sl_walks<false><<<grid_for((const void*)k_sl_walks<false>, threads, 0, work), threads, 0, s>>>(p);
+            k_sl_walks_ris<false><<<grid_for((const void*)k_sl_walks_ris<false>, threads, 0, work), threads, 0, s>>>(p);
     } else if (debug) {
         k_sl_walks_ff<true><<<grid_for((const void*)k_sl_walks_ff<true>, threads, 0, work), threads, 0, s>>>(p);
     } else {
