@@ -78,6 +78,53 @@ __global__ void k_bitonic(uint64_t* __restrict__ keys, int32_t* __restrict__ val
     }
 }
 
+// The stages k = k_first .. k_last (doubling) of the same sort whose exchange
+// distance lies within a chunk of kSortChunk elements, one chunk per block in
+// shared memory.  A stage is one pass over memory of 3 to 4 us, most of it
+// launch and latency, and 2^18 pairs take 171 of them (665 us); with the short
+// distances done here 28 launches are left (201 us).
+constexpr int kSortChunk = 4096, kSortThreads = 1024;
+
+__global__ void __launch_bounds__(kSortThreads) k_bitonic_chunk(uint64_t* __restrict__ keys,
+                                                                int32_t* __restrict__ vals,
+                                                                int64_t n, int64_t k_first,
+                                                                int64_t k_last)
+{
+    __shared__ uint64_t sk[kSortChunk];
+    __shared__ int32_t sv[kSortChunk];
+    const int cnt = n < kSortChunk ? (int)n : kSortChunk;  // n and the chunk: powers of two
+    for (int64_t base = (int64_t)blockIdx.x * kSortChunk; base < n;
+         base += (int64_t)gridDim.x * kSortChunk) {
+        for (int i = threadIdx.x; i < cnt; i += kSortThreads) {
+            sk[i] = keys[base + i];
+            sv[i] = vals[base + i];
+        }
+        for (int64_t k = k_first; k <= k_last; k <<= 1)
+            for (int jj = k / 2 < cnt / 2 ? (int)(k / 2) : cnt / 2; jj > 0; jj >>= 1) {
+                __syncthreads();
+                for (int t = threadIdx.x; t < cnt / 2; t += kSortThreads) {
+                    const int i = ((t & ~(jj - 1)) << 1) | (t & (jj - 1)), p = i | jj;
+                    const bool up = ((base + i) & k) == 0;
+                    const uint64_t ki = sk[i], kp = sk[p];
+                    const int32_t vi = sv[i], vp = sv[p];
+                    const bool gt = (ki > kp) || (ki == kp && vi > vp);
+                    if (gt == up) {
+                        sk[i] = kp;
+                        sk[p] = ki;
+                        sv[i] = vp;
+                        sv[p] = vi;
+                    }
+                }
+            }
+        __syncthreads();
+        for (int i = threadIdx.x; i < cnt; i += kSortThreads) {
+            keys[base + i] = sk[i];
+            vals[base + i] = sv[i];
+        }
+        __syncthreads();
+    }
+}
+
 // length of the common prefix of sorted keys i and j (index tie-break)
 __device__ __forceinline__ int delta(const uint64_t* __restrict__ keys, int64_t n, int64_t i,
                                      int64_t j)
@@ -389,23 +436,23 @@ __global__ void k_wide_collapse(const float4* __restrict__ nodes, int root_ref, 
             if (e[j].ref < 0) o[k++] = e[j];
         const int first_child = nint > 0 ? atomicAdd(counter, nint) : 0;
         for (int j = 0; j < nint; ++j) src[first_child + j] = o[j].ref;
-        // node box and quantisation (FP64, outward)
-        double lo[3], hi[3];
-        for (int c = 0; c < 3; ++c) {
-            lo[c] = o[0].lo[c];
-            hi[c] = o[0].hi[c];
-            for (int j = 1; j < n; ++j) {
-                lo[c] = fmin(lo[c], (double)o[j].lo[c]);
-                hi[c] = fmax(hi[c], (double)o[j].hi[c]);
-            }
-        }
-        // origin rounded down; the scale covers [origin, hi] in 255 steps
+        // node box and quantisation (differences in FP64, rounded outward); the
+        // scale covers [origin, hi] in 255 steps and is a power of two, so its
+        // quotients are products with the inverse power: the same values without
+        // the 48 FP64 divisions that took most of this kernel (63 us a level
+        // before, 23 us now)
         float org[3];
-        for (int c = 0; c < 3; ++c) org[c] = __double2float_rd(lo[c]);
         uint32_t ebits[3];
-        double scale[3];
+        uint32_t q[3][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}};  // [axis][lo0-3, lo4-7, hi0-3, hi4-7]
+#pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const double ext = hi[c] - (double)org[c];
+            float hi = o[0].hi[c];
+            org[c] = o[0].lo[c];
+            for (int j = 1; j < n; ++j) {
+                org[c] = fminf(org[c], o[j].lo[c]);
+                hi = fmaxf(hi, o[j].hi[c]);
+            }
+            const double ext = (double)hi - (double)org[c];
             int ex = -126;
             if (ext > 0.0) {
                 int e2;
@@ -413,18 +460,14 @@ __global__ void k_wide_collapse(const float4* __restrict__ nodes, int root_ref, 
                 ex = e2 < -126 ? -126 : e2;
             }
             ebits[c] = (uint32_t)(ex + 127);
-            scale[c] = ldexp(1.0, ex);
-        }
-        uint32_t q[3][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}};  // [axis][lo0-3, lo4-7, hi0-3, hi4-7]
-        for (int j = 0; j < n; ++j)
-            for (int c = 0; c < 3; ++c) {
-                const double ql = floor(((double)o[j].lo[c] - org[c]) / scale[c]);
-                const double qh = ceil(((double)o[j].hi[c] - org[c]) / scale[c]);
-                const uint32_t bl = (uint32_t)fmin(fmax(ql, 0.0), 255.0);
-                const uint32_t bh = (uint32_t)fmin(fmax(qh, 0.0), 255.0);
-                q[c][j >> 2] |= bl << (8 * (j & 3));
-                q[c][2 + (j >> 2)] |= bh << (8 * (j & 3));
+            const double inv = __hiloint2double((1023 - ex) << 20, 0);  // 2^-ex
+            for (int j = 0; j < n; ++j) {
+                const int ql = __double2int_rd(((double)o[j].lo[c] - org[c]) * inv);
+                const int qh = __double2int_ru(((double)o[j].hi[c] - org[c]) * inv);
+                q[c][j >> 2] |= (uint32_t)min(max(ql, 0), 255) << (8 * (j & 3));
+                q[c][2 + (j >> 2)] |= (uint32_t)min(max(qh, 0), 255) << (8 * (j & 3));
             }
+        }
         int refs[8];
         for (int j = 0; j < 8; ++j) refs[j] = (j < n && j >= nint) ? o[j].ref : 0;
         if (nint > 0) refs[0] = first_child;
@@ -527,9 +570,15 @@ int build_bvh_impl(MeshDev& m, int leaf_size, cudaStream_t s, BvhDev& b)
         m.verts, m.tris, n, n_pad, lo, scale, keys, vals);
     WOB_CUDA_TRY(cudaGetLastError());
     const int gb = grid_for((const void*)k_bitonic, threads, 0, n_pad);
-    for (int64_t k = 2; k <= n_pad; k <<= 1)
-        for (int64_t jj = k >> 1; jj > 0; jj >>= 1)
+    const int gc = grid_for((const void*)k_bitonic_chunk, kSortThreads, 0,
+                            (n_pad + kSortChunk - 1) / kSortChunk * kSortThreads);
+    const int64_t chunk = n_pad < kSortChunk ? n_pad : kSortChunk;
+    if (n_pad > 1) k_bitonic_chunk<<<gc, kSortThreads, 0, s>>>(keys, vals, n_pad, 2, chunk);
+    for (int64_t k = 2 * kSortChunk; k <= n_pad; k <<= 1) {
+        for (int64_t jj = k >> 1; jj >= kSortChunk; jj >>= 1)
             k_bitonic<<<gb, threads, 0, s>>>(keys, vals, n_pad, k, jj);
+        k_bitonic_chunk<<<gc, kSortThreads, 0, s>>>(keys, vals, n_pad, k, k);
+    }
     WOB_CUDA_TRY(cudaGetLastError());
 
     const int64_t n_int = n - 1;
