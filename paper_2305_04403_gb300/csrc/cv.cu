@@ -45,8 +45,8 @@ struct CvGeom {
     const float4* tri_c;         // centroid, near radius (near x longest edge)
     const float4* tri_p;         // unit normal n, plane offset n . y of the triangle
     const float* tri_a;          // area
-    const float4* coarse_pk;     // T x 7: position, weight x node value (paired, k_cv_pack)
-    const float4* fine_pk;       // T x F, the same layout
+    const float4* far;           // triangles and coarse nodes, two triangles per record (kFarRec)
+    const float4* fine_pk;       // T x F: position, weight x node value (paired, k_cv_pack)
     const int* cand_off;         // per triangle: candidate near triangles
     const int* cand;
 };
@@ -98,12 +98,29 @@ void rule_tables(int level, std::vector<float>& cb, std::vector<float>& cw,
         }
 }
 
+// Far-field records: what the far field reads of a triangle, two triangles to
+// a record, slot i of either at floats 2 i and 2 i + 1 -- the lanes of packed
+// FP32x2 operations, so that all of a triangle's arithmetic is packed (pairs
+// of its 7 nodes left the odd node, the plane and the near test scalar).  The
+// missing partner of an odd last triangle is near to every point, so nothing
+// of it counts.
+constexpr int kFarC = 0, kFarNear2 = 3, kFarN = 4, kFarOff = 7, kFarNode = 8,  // 7 x (x, y, z, w f)
+              kFarArea = kFarNode + 4 * kCoarse;
+constexpr int kFarRec = (kFarArea + 2) / 2;  // float4 per record (the last half unused)
+
+__device__ __forceinline__ float* far_slot(float4* far, int64_t j, int slot)
+{
+    return reinterpret_cast<float*>(far + (j >> 1) * kFarRec) + 2 * slot + (j & 1);
+}
+
 __global__ void k_cv_nodes(const float* __restrict__ verts, const int32_t* __restrict__ tris,
                            int T, int F, float near, float4* __restrict__ tri_c,
                            float4* __restrict__ tri_p, float* __restrict__ tri_R,
                            float* __restrict__ tri_a, float4* __restrict__ coarse,
-                           float4* __restrict__ fine)
+                           float4* __restrict__ fine, float4* __restrict__ far)
 {
+    if ((T & 1) && blockIdx.x == 0 && threadIdx.x < 2 * kFarRec)
+        *far_slot(far, T, threadIdx.x) = threadIdx.x == kFarNear2 ? INFINITY : 0.f;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < T; j += gridDim.x * blockDim.x) {
         double v[3][3];
         for (int k = 0; k < 3; ++k)
@@ -132,6 +149,13 @@ __global__ void k_cv_nodes(const float* __restrict__ verts, const int32_t* __res
                                (float)(n[0] * cen[0] + n[1] * cen[1] + n[2] * cen[2]));
         tri_R[j] = (float)R;
         tri_a[j] = (float)area;
+        for (int c = 0; c < 3; ++c) {
+            *far_slot(far, j, kFarC + c) = (float)cen[c];
+            *far_slot(far, j, kFarN + c) = (float)n[c];
+        }
+        *far_slot(far, j, kFarNear2) = (float)(near * h) * (float)(near * h);
+        *far_slot(far, j, kFarOff) = tri_p[j].w;
+        *far_slot(far, j, kFarArea) = (float)area;
         for (int q = 0; q < kCoarse; ++q) {
             double p[3];
             for (int c = 0; c < 3; ++c)
@@ -139,6 +163,7 @@ __global__ void k_cv_nodes(const float* __restrict__ verts, const int32_t* __res
                        c_coarse_b[3 * q + 2] * v[2][c];
             coarse[kCoarse * j + q] = make_float4((float)p[0], (float)p[1], (float)p[2],
                                                   (float)(c_coarse_w[q] * area));
+            for (int c = 0; c < 3; ++c) *far_slot(far, j, kFarNode + 4 * q + c) = (float)p[c];
         }
         for (int q = 0; q < F; ++q) {
             double p[3];
@@ -149,6 +174,15 @@ __global__ void k_cv_nodes(const float* __restrict__ verts, const int32_t* __res
                                                    (float)(c_fine_w[q] * area));
         }
     }
+}
+
+// Weight x value of the coarse nodes into the far-field records.
+__global__ void k_cv_pack_far(const float4* __restrict__ nodes, const float* __restrict__ val,
+                              int64_t n, float4* __restrict__ far)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x)
+        *far_slot(far, i / kCoarse, kFarNode + 4 * (int)(i % kCoarse) + 3) = nodes[i].w * val[i];
 }
 
 // Packed nodes for the sums: position and weight x value, `per` nodes per
@@ -200,10 +234,12 @@ __global__ void k_cv_candidates(int T, const float4* __restrict__ tri_c,
     }
 }
 
+// Whether the triangle's fine nodes are taken for x.  The far field makes the
+// same decision: the same operations in the same order.
 __device__ __forceinline__ bool is_near(float4 tc, float3 x)
 {
     const float dx = tc.x - x.x, dy = tc.y - x.y, dz = tc.z - x.z;
-    return dx * dx + dy * dy + dz * dz < tc.w * tc.w;
+    return fmaf(dz, dz, fmaf(dx, dx, dy * dy)) < tc.w * tc.w;
 }
 
 // One node: t = 1/r^3, r = |y - x|; s1 += (w f) t, s0 += omega t (omega: the
@@ -220,11 +256,11 @@ __device__ __forceinline__ void node_acc(float4 nd, float omega, float3 x, float
 // node_acc for two nodes at once, stored as (x, x', y, y'), (z, z', w, w'):
 // packed FP32x2 operations, every lane rounded as node_acc rounds it (r =
 // node - x as node + (-x)).
-static_assert(kCoarse % 2 == 1, "coarse nodes: pairs plus one");
 struct NegPoint2 {
     float2 x, y, z;  // (-x, -x), ...
 };
 
+template <bool VALUE = true>
 __device__ __forceinline__ void node_acc2(float4 a, float4 b, float2 omega, const NegPoint2& nx,
                                           float2& s1, float2& s0)
 {
@@ -235,164 +271,292 @@ __device__ __forceinline__ void node_acc2(float4 a, float4 b, float2 omega, cons
     const float2 ri = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
     const float2 t = __fmul2_rn(__fmul2_rn(ri, ri), ri);
     s1 = __ffma2_rn(make_float2(b.z, b.w), t, s1);
-    s0 = __ffma2_rn(omega, t, s0);
+    if (VALUE) s0 = __ffma2_rn(omega, t, s0);
 }
 
 // On the flat triangle j every node has the same r . n_j = d_j - x . n_j, so
 //   sum_q w_q (r . n)/r^3 (f_q - fx) = (d_j - x . n_j) (S1 - fx area_j S0),
+// added to `sum` with one rounding,
 // S1 = sum_q (w_q f_q) / r_q^3, S0 = sum_q omega_q / r_q^3 (w_q = area_j omega_q).
 __device__ __forceinline__ float tri_term(float4 tp, float area, float3 x, float fx, float s1,
-                                          float s0)
+                                          float s0, float sum)
 {
     const float dot = tp.w - fmaf(x.x, tp.x, fmaf(x.y, tp.y, x.z * tp.z));
-    return dot * fmaf(-fx * area, s0, s1);
+    return fmaf(dot, fmaf(-fx * area, s0, s1), sum);
 }
 
-// Far-field tile: kTileTris triangles (centroid + near radius, plane, area)
-// and their packed coarse nodes (paired layout, see k_cv_pack), staged in
-// shared memory by the whole block.
-constexpr int kQuadThreads = 256;
+// Far-field tile: kTileTris triangles' records, staged in shared memory by the
+// whole block.
+constexpr int kQuadThreads = 128;
 constexpr int kTileTris = 64;
 // Near-field stage: the fine nodes of up to kNearStage / F candidate
 // triangles (at least one: F <= kMaxFine <= kNearStage).
 constexpr int kNearStage = 512;
 static_assert(kMaxFine <= kNearStage, "one triangle's fine nodes fit the stage");
 struct FarTile {
-    float4 tc[kTileTris];
-    float4 tp[kTileTris];
-    float ta[kTileTris];
-    float4 node[kTileTris * kCoarse];
+    float4 rec[kTileTris / 2 * kFarRec];
     float4 fine[kNearStage];
     int own0;
 };
+static_assert(kTileTris % 2 == 0, "records hold two triangles");
 
-// Fine-node sum of triangle j (its 4^level sub-triangles) from its F nodes
-// at nd: global memory (read-only path) or a block's shared-memory stage.
+// `sum` plus the fine-node sum of triangle j (its 4^level sub-triangles) from its F nodes
+// at nd: global memory (read-only path) or a block's shared-memory stage.  Two
+// sub-triangles (seven pairs) are one turn: the rule's weights repeat, so they
+// stay in registers (an indexed constant load per pair otherwise), and their
+// loads are in flight together.
 template <bool SHARED>
 __device__ __forceinline__ float fine_sum(const CvGeom& c, const float4* nd, int j, float3 x,
-                                          float fx)
+                                          float fx, float sum)
 {
+    const float4 tp = __ldg(c.tri_p + j);
+    const float area = __ldg(c.tri_a + j);
     const NegPoint2 nx{make_float2(-x.x, -x.x), make_float2(-x.y, -x.y), make_float2(-x.z, -x.z)};
     float2 s1p = make_float2(0.f, 0.f), s0p = make_float2(0.f, 0.f);
-    const int pairs = c.F >> 1;
-#pragma unroll 4  // four pairs' loads in flight (the far loop unrolled too runs slower)
-    for (int q = 0; q < pairs; ++q)
+    auto pair = [&](int q, float2 om) {
         node_acc2(SHARED ? nd[2 * q] : __ldg(nd + 2 * q), SHARED ? nd[2 * q + 1] : __ldg(nd + 2 * q + 1),
-                  make_float2(c_fine_w[2 * q], c_fine_w[2 * q + 1]), nx, s1p, s0p);
-    float s1 = s1p.x + s1p.y, s0 = s0p.x + s0p.y;
-    if (c.F & 1) node_acc(SHARED ? nd[c.F - 1] : __ldg(nd + c.F - 1), c_fine_w[c.F - 1], x, s1, s0);
-    return tri_term(__ldg(c.tri_p + j), __ldg(c.tri_a + j), x, fx, s1, s0);
+                  om, nx, s1p, s0p);
+    };
+    if (c.F == kCoarse) {  // level 0: one triangle, three pairs and the odd node
+#pragma unroll
+        for (int q = 0; q < kCoarse / 2; ++q) pair(q, make_float2(c_fine_w[2 * q], c_fine_w[2 * q + 1]));
+        float s1 = s1p.x + s1p.y, s0 = s0p.x + s0p.y;
+        node_acc(SHARED ? nd[c.F - 1] : __ldg(nd + c.F - 1), c_fine_w[kCoarse - 1], x, s1, s0);
+        return tri_term(tp, area, x, fx, s1, s0, sum);
+    }
+    const float w0 = c_fine_w[0], w1 = c_fine_w[1], w2 = c_fine_w[4];  // centroid, orbits
+    for (int g = 0; g < c.F; g += 2 * kCoarse, nd += 2 * kCoarse) {
+        pair(0, make_float2(w0, w1));
+        pair(1, make_float2(w1, w1));
+        pair(2, make_float2(w2, w2));
+        pair(3, make_float2(w2, w0));
+        pair(4, make_float2(w1, w1));
+        pair(5, make_float2(w1, w2));
+        pair(6, make_float2(w2, w2));
+    }
+    return tri_term(tp, area, x, fx, s1p.x + s1p.y, s0p.x + s0p.y, sum);
 }
 
-__device__ __forceinline__ float fine_tri(const CvGeom& c, int j, float3 x, float fx)
+__device__ __forceinline__ float fine_tri(const CvGeom& c, int j, float3 x, float fx, float sum)
 {
-    return fine_sum<false>(c, c.fine_pk + (int64_t)c.F * j, j, x, fx);
+    return fine_sum<false>(c, c.fine_pk + (int64_t)c.F * j, j, x, fx, sum);
+}
+
+// Far field of the two triangles of a record: their terms (tri_term of the
+// coarse nodes' sums) for x, and whether either is near.  Every lane is
+// rounded as the scalar operations round it, nodes 0, 2, 4 and 1, 3, 5 in two
+// sums that meet before node 6.  VALUE: fx counts (else 0, and S0 is not formed).
+// Bounded by the FMA pipe: 80 packed operations (two cycles each) for 63
+// instructions a triangle, 3.6 of the 9.5 -> 7.46 ms that the residual walks of
+// 8,192 queries x 64 walks x 2 vertices take (fine nodes 2.6).  A form with the
+// centroid's distance and offsets along two medians needs 30% fewer operations,
+// and rounds differently.
+template <bool VALUE>
+__device__ __forceinline__ float2 far_pair(const float4* t, const float (&om)[kCoarse],
+                                           const NegPoint2& nx, float fx, bool& near0, bool& near1)
+{
+    auto lo = [](float4 v) { return make_float2(v.x, v.y); };
+    auto hi = [](float4 v) { return make_float2(v.z, v.w); };
+    auto dup = [](float v) { return make_float2(v, v); };
+    const float4 c0 = t[0], c1 = t[1];
+    const float2 dx = __fadd2_rn(lo(c0), nx.x), dy = __fadd2_rn(hi(c0), nx.y),
+                 dz = __fadd2_rn(lo(c1), nx.z);
+    const float2 d2 = __ffma2_rn(dz, dz, __ffma2_rn(dx, dx, __fmul2_rn(dy, dy)));
+    near0 = d2.x < c1.z;
+    near1 = d2.y < c1.w;
+    float2 s1[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    float2 s0[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+    for (int q = 0; q < kCoarse; ++q) {
+        if (q == kCoarse - 1) {
+            s1[0] = __fadd2_rn(s1[0], s1[1]);
+            s0[0] = __fadd2_rn(s0[0], s0[1]);
+        }
+        node_acc2<VALUE>(t[kFarNode / 2 + 2 * q], t[kFarNode / 2 + 2 * q + 1], dup(om[q]), nx,
+                         s1[q & 1], s0[q & 1]);
+    }
+    const float4 p0 = t[kFarN / 2], p1 = t[kFarN / 2 + 1];
+    const float2 xn = __ffma2_rn(nx.x, lo(p0), __ffma2_rn(nx.y, hi(p0), __fmul2_rn(nx.z, lo(p1))));
+    const float2 dot = __fadd2_rn(hi(p1), xn);
+    if (!VALUE) return __fmul2_rn(dot, s1[0]);
+    return __fmul2_rn(dot, __ffma2_rn(__fmul2_rn(dup(-fx), lo(t[kFarArea / 2])), s0[0], s1[0]));
 }
 
 // sum over quadrature nodes of w (r . n)/(4 pi r^3) (f(y) - fx), r = y - x,
-// i.e. -int dG/dn_y (f - fx) dA, skipping triangle `own` (-1: none).
+// i.e. -int dG/dn_y (f - fx) dA, for a point of triangle `own`, which is skipped.
 // Called by EVERY thread of the block (the triangle tiles and the near
-// field's fine nodes are loaded cooperatively); `own` must be negative for
-// all threads of the block or for none.  The far field (coarse nodes of every triangle not near x) is an
-// N-body sum over shared-memory tiles, FP32 within a tile and FP64 across
-// tiles.  Near triangles (fine nodes): per lane from the candidate list of
-// `own` when own >= 0; otherwise decided per triangle for the whole warp.
+// field's fine nodes are loaded cooperatively).  The far field (coarse nodes of
+// every triangle not near x) is an N-body sum over shared-memory tiles, FP32
+// within a tile and FP64 across tiles.  Near triangles (fine nodes): per lane
+// from the candidate list of `own`.
 __device__ __forceinline__ float quad_sum(const CvGeom& c, FarTile& sm, float3 x, int own,
                                           float fx)
 {
     double tot = 0.0;
-    // the coarse weights of the node pairs and the negated query, in registers
-    float2 om[(kCoarse - 1) / 2];
+    // the coarse weights and the negated query, in registers
+    float om[kCoarse];
 #pragma unroll
-    for (int q = 0; q < (kCoarse - 1) / 2; ++q)
-        om[q] = make_float2(c_coarse_w[2 * q], c_coarse_w[2 * q + 1]);
-    const float om_last = c_coarse_w[kCoarse - 1];
+    for (int q = 0; q < kCoarse; ++q) om[q] = c_coarse_w[q];
     const NegPoint2 nx{make_float2(-x.x, -x.x), make_float2(-x.y, -x.y), make_float2(-x.z, -x.z)};
     for (int j0 = 0; j0 < c.T; j0 += kTileTris) {
         const int nt = min(kTileTris, c.T - j0);
+        const int n = ((nt + 1) >> 1) * kFarRec;
         __syncthreads();  // the previous tile is no longer read
-        for (int i = threadIdx.x; i < nt; i += blockDim.x) {
-            sm.tc[i] = __ldg(c.tri_c + j0 + i);
-            sm.tp[i] = __ldg(c.tri_p + j0 + i);
-            sm.ta[i] = __ldg(c.tri_a + j0 + i);
-        }
-        for (int i = threadIdx.x; i < nt * kCoarse; i += blockDim.x)
-            sm.node[i] = __ldg(c.coarse_pk + (int64_t)kCoarse * j0 + i);
+        for (int i = threadIdx.x; i < n; i += blockDim.x)
+            sm.rec[i] = __ldg(c.far + (int64_t)(j0 >> 1) * kFarRec + i);
         __syncthreads();
         float part = 0.f;
-        for (int jj = 0; jj < nt; ++jj) {
+        for (int jj = 0; jj < nt; jj += 2) {
             const int j = j0 + jj;
-            const bool near_me = is_near(sm.tc[jj], x);
-            const float4* nb = sm.node + kCoarse * jj;
-            float2 s1p = make_float2(0.f, 0.f), s0p = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int q = 0; q < (kCoarse - 1) / 2; ++q)
-                node_acc2(nb[2 * q], nb[2 * q + 1], om[q], nx, s1p, s0p);
-            float s1 = s1p.x + s1p.y, s0 = s0p.x + s0p.y;
-            node_acc(nb[kCoarse - 1], om_last, x, s1, s0);
-            const float term = tri_term(sm.tp[jj], sm.ta[jj], x, fx, s1, s0);
-            part += (j == own || near_me) ? 0.f : term;
-            if (own < 0 && __any_sync(0xFFFFFFFFu, near_me)) {
-                const float fterm = fine_tri(c, j, x, fx);
-                part += near_me ? fterm : 0.f;
-            }
+            bool near0, near1;
+            const float2 term =
+                far_pair<true>(sm.rec + (jj >> 1) * kFarRec, om, nx, fx, near0, near1);
+            part += (j == own || near0) ? 0.f : term.x;
+            part += (j + 1 == own || near1) ? 0.f : term.y;
         }
         tot += (double)part;
     }
-    if (own >= 0) {
-        float near_tot = 0.f;
-        __syncthreads();  // the last far tile is no longer read
-        if (threadIdx.x == 0) sm.own0 = own;
-        __syncthreads();
-        if (__syncthreads_and(own == sm.own0)) {
-            // the whole block shares the triangle (the walks are bucketed by
-            // it): its candidates' fine nodes are staged in shared memory,
-            // chunk by chunk, and read by every lane as broadcasts; the
-            // candidates are visited in the same order as below
-            const int beg = own == 0 ? 0 : c.cand_off[own - 1], end = c.cand_off[own];
-            const int per = kNearStage / c.F;
-            for (int c0 = beg; c0 < end; c0 += per) {
-                const int nt = min(per, end - c0);
-                __syncthreads();  // the previous chunk is no longer read
-                for (int i = threadIdx.x; i < nt * c.F; i += blockDim.x)
-                    sm.fine[i] = __ldg(c.fine_pk + (int64_t)c.F * c.cand[c0 + i / c.F] + i % c.F);
-                __syncthreads();
-                for (int k = 0; k < nt; ++k) {
-                    const int j = c.cand[c0 + k];
-                    if (is_near(__ldg(c.tri_c + j), x))
-                        near_tot += fine_sum<true>(c, sm.fine + k * c.F, j, x, fx);
-                }
-            }
-        } else {
-            for (int ci = own == 0 ? 0 : c.cand_off[own - 1]; ci < c.cand_off[own]; ++ci) {
-                const int j = c.cand[ci];
-                if (is_near(__ldg(c.tri_c + j), x)) near_tot += fine_tri(c, j, x, fx);
+    float near_tot = 0.f;
+    __syncthreads();  // the last far tile is no longer read
+    if (threadIdx.x == 0) sm.own0 = own;
+    __syncthreads();
+    if (__syncthreads_and(own == sm.own0)) {
+        // the whole block shares the triangle (the walks are bucketed by
+        // it): its candidates' fine nodes are staged in shared memory,
+        // chunk by chunk, and read by every lane as broadcasts; the
+        // candidates are visited in the same order as below
+        const int beg = own == 0 ? 0 : c.cand_off[own - 1], end = c.cand_off[own];
+        const int per = kNearStage / c.F;
+        for (int c0 = beg; c0 < end; c0 += per) {
+            const int nt = min(per, end - c0);
+            __syncthreads();  // the previous chunk is no longer read
+            for (int i = threadIdx.x; i < nt * c.F; i += blockDim.x)
+                sm.fine[i] = __ldg(c.fine_pk + (int64_t)c.F * c.cand[c0 + i / c.F] + i % c.F);
+            __syncthreads();
+            for (int k = 0; k < nt; ++k) {
+                const int j = c.cand[c0 + k];
+                if (is_near(__ldg(c.tri_c + j), x))
+                    near_tot = fine_sum<true>(c, sm.fine + k * c.F, j, x, fx, near_tot);
             }
         }
-        tot += (double)near_tot;
+    } else {
+        for (int ci = own == 0 ? 0 : c.cand_off[own - 1]; ci < c.cand_off[own]; ++ci) {
+            const int j = c.cand[ci];
+            if (is_near(__ldg(c.tri_c + j), x)) near_tot = fine_tri(c, j, x, fx, near_tot);
+        }
     }
+    tot += (double)near_tot;
     return (float)(tot * (double)kInvFourPi);
 }
 
-// (D f)(x0) at points off the surface: -quad_sum(f) with f(x) = 0.
-__global__ void __launch_bounds__(kQuadThreads, 4) k_cv_quad_D(CvGeom c, const float* __restrict__ x,
-                                                           int64_t n, float* out)
+// (D f)(x0) at points off the surface: the quadrature of quad_sum with
+// f(x) = 0 and no own triangle.  A block takes 32 points, lane = point, and its
+// warps share the triangles (16 records each of a staged tile), so that a call
+// of few points still fills the SMs.  Points off the surface have no candidate
+// list and the 32 of a warp lie anywhere: their (point, near triangle) pairs
+// are queued, and eight lanes sum the fine nodes of one pair.  Evaluating a
+// triangle's fine nodes for the whole warp whenever it is near to one lane took
+// 1,196 us at 8,192 points and 1,280 triangles (18 near to each point), most of
+// it for lanes that did not need them; this form 66 us.
+constexpr int kPointWarps = 8, kPointTris = 256, kPairQueue = 128, kPairLanes = 8;
+struct PointTile {
+    float4 rec[kPointTris / 2 * kFarRec];
+    int queue[kPointWarps][kPairQueue];  // lane << 20 | triangle
+    double sum[kPointWarps][32];
+};
+static_assert(sizeof(PointTile) <= 48 * 1024, "static shared memory");
+
+// The fine-node terms of `count` queued pairs, added to their lanes' sums.
+__device__ __forceinline__ void near_pairs(const CvGeom& c, const int* queue, int count, float3 x,
+                                           float& sum)
 {
-    __shared__ FarTile sm;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n;
-         base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = base + threadIdx.x;
+    const int lane = threadIdx.x & 31, sub = lane & (kPairLanes - 1), pairs = c.F >> 1;
+    __syncwarp();
+    for (int e0 = 0; e0 < count; e0 += 32 / kPairLanes) {
+        const int e = e0 + lane / kPairLanes;
+        const int entry = queue[e < count ? e : e0];
+        const int who = entry >> 20, j = entry & 0xFFFFF;
+        const float3 y = make_float3(__shfl_sync(0xFFFFFFFFu, x.x, who), __shfl_sync(0xFFFFFFFFu, x.y, who),
+                                     __shfl_sync(0xFFFFFFFFu, x.z, who));
+        const NegPoint2 ny{make_float2(-y.x, -y.x), make_float2(-y.y, -y.y), make_float2(-y.z, -y.z)};
+        const float4* nd = c.fine_pk + (int64_t)c.F * j;
+        float2 s1p = make_float2(0.f, 0.f), s0p = s1p;
+        for (int q = sub; q < pairs; q += kPairLanes)
+            node_acc2<false>(__ldg(nd + 2 * q), __ldg(nd + 2 * q + 1), s0p, ny, s1p, s0p);
+        float s1 = s1p.x + s1p.y, s0 = 0.f;
+        if ((c.F & 1) && sub == kPairLanes - 1) node_acc(__ldg(nd + c.F - 1), 0.f, y, s1, s0);
+        for (int o = kPairLanes / 2; o > 0; o >>= 1) s1 += __shfl_xor_sync(0xFFFFFFFFu, s1, o);
+        const float term = e < count ? tri_term(__ldg(c.tri_p + j), 0.f, y, 0.f, s1, 0.f, 0.f) : 0.f;
+        for (int g = 0; g < 32; g += kPairLanes) {
+            const float v = __shfl_sync(0xFFFFFFFFu, term, g);
+            if (lane == __shfl_sync(0xFFFFFFFFu, who, g)) sum += v;
+        }
+    }
+    __syncwarp();
+}
+
+__global__ void __launch_bounds__(32 * kPointWarps) k_cv_quad_D(CvGeom c, const float* __restrict__ x,
+                                                                int64_t n, float* out)
+{
+    __shared__ PointTile sm;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int kShare = kPointTris / 2 / kPointWarps;  // records of a tile per warp
+    const float om[kCoarse] = {};
+    int* queue = sm.queue[warp];
+    for (int64_t base = 32 * (int64_t)blockIdx.x; base < n; base += 32 * (int64_t)gridDim.x) {
+        const int64_t i = base + lane;
         const bool ok = i < n;
         const float3 p = ok ? make_float3(x[3 * i], x[3 * i + 1], x[3 * i + 2])
                             : make_float3(0.f, 0.f, 0.f);
-        const float v = quad_sum(c, sm, p, -1, 0.f);
-        if (ok) out[i] = v;
+        const NegPoint2 nx{make_float2(-p.x, -p.x), make_float2(-p.y, -p.y), make_float2(-p.z, -p.z)};
+        double tot = 0.0;
+        float near_tot = 0.f;
+        int queued = 0;
+        for (int j0 = 0; j0 < c.T; j0 += kPointTris) {
+            const int recs = (min(kPointTris, c.T - j0) + 1) >> 1;
+            __syncthreads();  // the previous tile is no longer read
+            for (int k = threadIdx.x; k < recs * kFarRec; k += blockDim.x)
+                sm.rec[k] = __ldg(c.far + (int64_t)(j0 >> 1) * kFarRec + k);
+            __syncthreads();
+            float part = 0.f;
+            const int end = min(recs, (warp + 1) * kShare);
+            for (int r = warp * kShare; r < end; ++r) {
+                const int j = j0 + 2 * r;
+                bool near0, near1;
+                const float2 term = far_pair<false>(sm.rec + r * kFarRec, om, nx, 0.f, near0, near1);
+                part += near0 ? 0.f : term.x;
+                part += near1 ? 0.f : term.y;
+                near0 = near0 && ok;
+                near1 = near1 && ok && j + 1 < c.T;
+                if (__any_sync(0xFFFFFFFFu, near0 || near1)) {
+                    const unsigned b0 = __ballot_sync(0xFFFFFFFFu, near0),
+                                   b1 = __ballot_sync(0xFFFFFFFFu, near1), below = (1u << lane) - 1;
+                    if (near0) queue[queued + __popc(b0 & below)] = lane << 20 | j;
+                    queued += __popc(b0);
+                    if (near1) queue[queued + __popc(b1 & below)] = lane << 20 | (j + 1);
+                    queued += __popc(b1);
+                    if (queued > kPairQueue - 64) {
+                        near_pairs(c, queue, queued, p, near_tot);
+                        queued = 0;
+                    }
+                }
+            }
+            tot += (double)part;
+        }
+        near_pairs(c, queue, queued, p, near_tot);
+        sm.sum[warp][lane] = tot + (double)near_tot;
+        __syncthreads();
+        if (warp == 0 && ok) {
+            for (int k = 1; k < kPointWarps; ++k) tot = k == 1 ? sm.sum[0][lane] + sm.sum[1][lane] : tot + sm.sum[k][lane];
+            out[i] = (float)(tot * (double)kInvFourPi);
+        }
+        __syncthreads();
     }
 }
 
 // (H f)(x) at points on triangles prims (original ids): 2 phi int dG/dn_y f
 // = -2 phi quad_sum(f - f(x)) - phi f(x).
-__global__ void __launch_bounds__(kQuadThreads) k_cv_quad_H(CvGeom c, int phi,
+__global__ void __launch_bounds__(kQuadThreads, 8) k_cv_quad_H(CvGeom c, int phi,
                                                            const float* __restrict__ x,
                                                            const int32_t* __restrict__ prims,
                                                            const float* __restrict__ fx,
@@ -530,9 +694,11 @@ __global__ void k_cvw_scatter(CvWalk st)
 
 // Source r = 2 phi g - nu_t + H nu_t at the vertex reached at step k,
 // halved on the last vertex (Sec. 4.1.2), times the weight product.
-// 4 blocks of 256 per SM: 64 registers without spills (the compiler's own
-// choice, 48 registers and 5 blocks, spilled and ran 2.4% slower).
-__global__ void __launch_bounds__(kQuadThreads, 4) k_cvw_accum(WalkParams p, CvWalk st, CvGeom c,
+// 8 blocks of 128 per SM: 64 registers without spills (a block of 256 spans two
+// triangles' walks more often and runs 1.3% slower; the compiler's own 48
+// registers spilled, 2.4% slower; two points per thread halved the shared-memory
+// reads but left 12 to 24 warps an SM, 0.5 to 7% slower).
+__global__ void __launch_bounds__(kQuadThreads, 8) k_cvw_accum(WalkParams p, CvWalk st, CvGeom c,
                                                            int k)
 {
     __shared__ FarTile sm;
@@ -707,13 +873,13 @@ struct wob_cv_s {
     int T = 0, F = 0, level = 2;
     float near = 2.f;
     float4 *tri_c = nullptr, *tri_p = nullptr, *coarse = nullptr, *fine = nullptr;
-    float4 *coarse_pk = nullptr, *fine_pk = nullptr;
+    float4 *far = nullptr, *fine_pk = nullptr;
     float *tri_R = nullptr, *tri_a = nullptr, *coarse_val = nullptr, *fine_val = nullptr;
     int *cand_off = nullptr, *cand = nullptr;
     int64_t n_cand = 0;
     CvGeom geom() const
     {
-        return CvGeom{T, F, tri_c, tri_p, tri_a, coarse_pk, fine_pk, cand_off, cand};
+        return CvGeom{T, F, tri_c, tri_p, tri_a, far, fine_pk, cand_off, cand};
     }
 };
 
@@ -722,17 +888,25 @@ namespace {
 void free_cv(wob_cv_s* c)
 {
     for (void* p : {(void*)c->tri_c, (void*)c->tri_p, (void*)c->tri_R, (void*)c->tri_a,
-                    (void*)c->coarse, (void*)c->fine, (void*)c->coarse_pk, (void*)c->fine_pk,
+                    (void*)c->coarse, (void*)c->fine, (void*)c->far, (void*)c->fine_pk,
                     (void*)c->coarse_val, (void*)c->fine_val, (void*)c->cand_off, (void*)c->cand})
         if (p) cudaFree(p);
+}
+
+cudaError_t launch_quad_D(const CvGeom& g, const float* x, int64_t n, float* out, cudaStream_t s)
+{
+    const int threads = 32 * kPointWarps;
+    k_cv_quad_D<<<grid_for((const void*)k_cv_quad_D, threads, 0, n * kPointWarps), threads, 0, s>>>(
+        g, x, n, out);
+    return cudaGetLastError();
 }
 
 // Packed nodes from the current node values.
 int pack_nodes(wob_cv_s* c, cudaStream_t s)
 {
     const int64_t nc = (int64_t)c->T * kCoarse, nf = (int64_t)c->T * c->F;
-    k_cv_pack<<<grid_for((const void*)k_cv_pack, 256, 0, nc), 256, 0, s>>>(
-        c->coarse, c->coarse_val, nc, kCoarse, c->coarse_pk);
+    k_cv_pack_far<<<grid_for((const void*)k_cv_pack_far, 256, 0, nc), 256, 0, s>>>(
+        c->coarse, c->coarse_val, nc, c->far);
     k_cv_pack<<<grid_for((const void*)k_cv_pack, 256, 0, nf), 256, 0, s>>>(
         c->fine, c->fine_val, nf, c->F, c->fine_pk);
     WOB_CUDA_TRY(cudaGetLastError());
@@ -784,7 +958,7 @@ int wob_cv_create(wob_mesh m, int32_t level, float near, void* stream, wob_cv* o
         cudaMalloc((void**)&c->tri_a, T * sizeof(float)) != cudaSuccess ||
         cudaMalloc((void**)&c->coarse, (size_t)T * kCoarse * sizeof(float4)) != cudaSuccess ||
         cudaMalloc((void**)&c->fine, (size_t)T * c->F * sizeof(float4)) != cudaSuccess ||
-        cudaMalloc((void**)&c->coarse_pk, (size_t)T * kCoarse * sizeof(float4)) != cudaSuccess ||
+        cudaMalloc((void**)&c->far, (size_t)((T + 1) / 2) * kFarRec * sizeof(float4)) != cudaSuccess ||
         cudaMalloc((void**)&c->fine_pk, (size_t)T * c->F * sizeof(float4)) != cudaSuccess ||
         cudaMalloc((void**)&c->coarse_val, (size_t)T * kCoarse * sizeof(float)) != cudaSuccess ||
         cudaMalloc((void**)&c->fine_val, (size_t)T * c->F * sizeof(float)) != cudaSuccess ||
@@ -795,7 +969,7 @@ int wob_cv_create(wob_mesh m, int32_t level, float near, void* stream, wob_cv* o
     const int threads = 128;
     const int grid = grid_for((const void*)k_cv_nodes, threads, 0, T);
     k_cv_nodes<<<grid, threads, 0, s>>>(m->d.verts, m->d.tris, T, c->F, near, c->tri_c, c->tri_p,
-                                        c->tri_R, c->tri_a, c->coarse, c->fine);
+                                        c->tri_R, c->tri_a, c->coarse, c->fine, c->far);
     if (pack_nodes(c, s) != WOB_OK) return fail(WOB_ERR_CUDA, "node setup failed");
     int* count = nullptr;
     if (cudaMallocAsync((void**)&count, T * sizeof(int), s) != cudaSuccess)
@@ -865,9 +1039,7 @@ int wob_cv_quad_D(wob_cv c, const float* points, int64_t n, float* out, void* st
         return WOB_ERR_INVALID_ARG;
     }
     if (n == 0) return WOB_OK;
-    const int grid = grid_for((const void*)k_cv_quad_D, kQuadThreads, 0, n);
-    k_cv_quad_D<<<grid, kQuadThreads, 0, (cudaStream_t)stream>>>(c->geom(), points, n, out);
-    WOB_CUDA_TRY(cudaGetLastError());
+    WOB_CUDA_TRY(launch_quad_D(c->geom(), points, n, out, (cudaStream_t)stream));
     return WOB_OK;
 }
 
@@ -958,9 +1130,7 @@ int wob_cv_solve(const wob_problem* prob, wob_cv c, const float* params, const f
         if (cudaMemcpyAsync(per_walk, st.S, W * sizeof(double), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
             rc = WOB_ERR_CUDA;
     if (rc == WOB_OK && dnt) {
-        const int grid = grid_for((const void*)k_cv_quad_D, kQuadThreads, 0, Q);
-        k_cv_quad_D<<<grid, kQuadThreads, 0, s>>>(g, queries, Q, dnt);
-        if (cudaGetLastError() != cudaSuccess) rc = WOB_ERR_CUDA;
+        if (launch_quad_D(g, queries, Q, dnt, s) != cudaSuccess) rc = WOB_ERR_CUDA;
     }
     cudaFreeAsync(buf, s);
     if (rc != WOB_OK) set_error("wob_cv_solve failed");
