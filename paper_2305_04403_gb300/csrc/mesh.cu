@@ -113,14 +113,14 @@ __global__ void k_triangles(const float* __restrict__ verts, int64_t V,
         for (int c = 0; c < 3; ++c) {
             const double nc = n[c] / nl;
             fr.v0[c] = (float)a[c];
-            fr.e1h[c] = (float)e1[c];
-            fr.e1l[c] = (float)(e1[c] - (double)fr.e1h[c]);
-            fr.e2h[c] = (float)e2[c];
-            fr.e2l[c] = (float)(e2[c] - (double)fr.e2h[c]);
+            fr.eh[c][0] = (float)e1[c];
+            fr.el[c][0] = (float)(e1[c] - (double)fr.eh[c][0]);
+            fr.eh[c][1] = (float)e2[c];
+            fr.el[c][1] = (float)(e2[c] - (double)fr.eh[c][1]);
             fr.nh[c] = (float)nc;
             fr.nl[c] = (float)(nc - (double)fr.nh[c]);
-            fr.pad[c] = 0.f;
         }
+        fr.pad0 = fr.pad[0] = fr.pad[1] = 0.f;
         tri_f[j] = fr;
         // signed volume: a . (b x c) / 6
         vol += (a[0] * (b[1] * c[2] - b[2] * c[1]) + a[1] * (b[2] * c[0] - b[0] * c[2]) +

@@ -45,12 +45,11 @@ constexpr int kGroupBlocks = 24 / kG;
 // against 1,160 and 633 against 938 us; twice as many 226 against 205, 2,064
 // against 1,454 and 1,608 against 1,153 us.
 constexpr int64_t kGroupWalksPerSm = 200;
-// Single-layer walks with area sampling: 6 blocks of 128 threads per SM (71
-// registers, no spills) hide the latency of the CDF search better than the
-// unbounded 121 registers (4 blocks; 8% slower) or 8 blocks (64 registers,
-// spills; 3% slower).
+// Single-layer walks with area sampling: 7 blocks of 128 threads per SM (72
+// registers, no spills) hide the latency of the CDF search: 4.31 ms for 2.0e8
+// samples of the torus with 200,000 triangles, 4.51 with 6 blocks.
 #ifndef WOB_SL_MIN_BLOCKS
-#define WOB_SL_MIN_BLOCKS 6
+#define WOB_SL_MIN_BLOCKS 7
 #endif
 // Resampled single-layer walks: 7 blocks of 128 threads per SM (72 registers).  On
 // 1.05e6 walks of the mixed torus 6 blocks took 1.61 ms, 7 1.52, 8 (64 registers)
@@ -294,11 +293,11 @@ __device__ __forceinline__ int64_t area_pick(const WalkParams& p, uint32_t hi, u
     const uint64_t U = ((uint64_t)hi << 21) | (uint64_t)(lo >> 11);
     const long long target = __double_as_longlong(u53_unit(U) * p.area);
     const uint32_t b = hi >> (32 - p.guide_bits);  // top guide_bits bits of U
-    int64_t a = __ldg(p.guide + b);
-    int64_t e = __ldg(p.guide + b + 1);
-    e = e < p.T - 1 ? e : p.T - 1;
+    int32_t a = __ldg(p.guide + b), e = __ldg(p.guide + b + 1);
+    const int32_t last = (int32_t)p.T - 1;
+    e = e < last ? e : last;
     while (a < e) {
-        const int64_t mid = a + ((e - a) >> 1);
+        const int32_t mid = a + ((e - a) >> 1);
         if (__double_as_longlong(__ldg(p.cdf + mid)) > target) e = mid; else a = mid + 1;
     }
     return a;
@@ -319,6 +318,48 @@ __device__ __forceinline__ int64_t area_pick(const WalkParams& p, uint32_t hi, u
 // its bits by scale2) and the CDF target (one multiply).
 // ---------------------------------------------------------------------------
 
+// Two float-float values as the lanes of packed FP32x2 operations, each lane
+// rounded as ff.cuh's operations round it.  The low parts are kept negated (an
+// exact change): the packed operations take no negated operands, and the errors
+// come out of fma(a, -b, ab) and of differences without extra instructions.
+// Resampled walks 1.52 -> 1.38 ms against the scalar form (1.05e6 walks x 4
+// vertices x 16 candidates), single-layer walks, which wait for their loads
+// rather than for issue, 4.53 -> 4.51 ms.
+struct ff2 {
+    float2 hi, nlo;
+};
+__device__ __forceinline__ float2 sub2(float2 a, float2 b)
+{
+    return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
+}
+__device__ __forceinline__ ff2 two_sum2(float2 a, float2 b)
+{
+    const float2 s = __fadd2_rn(a, b), bb = sub2(s, a);
+    return {s, __fadd2_rn(sub2(sub2(s, bb), a), sub2(bb, b))};
+}
+__device__ __forceinline__ ff2 two_diff2(float2 a, float2 b)
+{
+    const float2 s = sub2(a, b), bb = sub2(s, a);
+    return {s, __fadd2_rn(sub2(sub2(s, bb), a), __fadd2_rn(bb, b))};
+}
+// fast_two_sum(a, -n)
+__device__ __forceinline__ ff2 fast_two_sub2(float2 a, float2 n)
+{
+    const float2 s = sub2(a, n);
+    return {s, __fadd2_rn(n, sub2(s, a))};
+}
+__device__ __forceinline__ ff2 ff_mul_f2(ff2 a, float2 b)
+{
+    const float2 nb = sub2(make_float2(0.f, 0.f), b), p = __fmul2_rn(a.hi, b);
+    return fast_two_sub2(p, __ffma2_rn(a.nlo, b, __ffma2_rn(a.hi, nb, p)));
+}
+// (ah + al) b
+__device__ __forceinline__ ff2 ff_mul2(float2 ah, float2 al, ff2 b)
+{
+    const float2 nb = sub2(make_float2(0.f, 0.f), b.hi), p = __fmul2_rn(ah, b.hi);
+    return fast_two_sub2(p, __ffma2_rn(ah, b.nlo, __ffma2_rn(al, nb, __ffma2_rn(ah, nb, p))));
+}
+
 // A boundary point in the compensated representation.
 struct FFPoint {
     float v0[3];  // the triangle's first vertex
@@ -335,29 +376,44 @@ __device__ __forceinline__ void frame_point_ff(const WalkParams& p, int64_t j, u
                                                uint32_t uw, FFPoint& y, float& b0, float& b1f,
                                                float& b2f)
 {
-    float fr[24];
     const float4* F = reinterpret_cast<const float4*>(p.tri_f + j);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        const float4 t = __ldg(F + i);
-        fr[4 * i] = t.x; fr[4 * i + 1] = t.y; fr[4 * i + 2] = t.z; fr[4 * i + 3] = t.w;
-    }
-    constexpr int o_e1h = offsetof(TriFrame, e1h) / 4, o_e1l = offsetof(TriFrame, e1l) / 4;
-    constexpr int o_e2h = offsetof(TriFrame, e2h) / 4, o_e2l = offsetof(TriFrame, e2l) / 4;
-    constexpr int o_nh = offsetof(TriFrame, nh) / 4, o_nl = offsetof(TriFrame, nl) / 4;
+    const float4 f0 = __ldg(F), f1 = __ldg(F + 1), f2 = __ldg(F + 2), f3 = __ldg(F + 3),
+                 f4 = __ldg(F + 4), f5 = __ldg(F + 5);
     const float u2 = u24f(uw);
     const ff su = ff_sqrt(u24f(uz));
-    const ff b1 = ff_mul_f(su, 1.f - u2), b2 = ff_mul_f(su, u2);
+    // (b1, b2) = sqrt(u1) (1 - u2, u2)
+    const ff2 b = ff_mul_f2({make_float2(su.hi, su.hi), make_float2(-su.lo, -su.lo)},
+                            make_float2(1.f - u2, u2));
     b0 = 1.f - su.hi;
-    b1f = b1.hi;
-    b2f = b2.hi;
+    b1f = b.hi.x;
+    b2f = b.hi.y;
+    const float2 eh[3] = {{f1.x, f1.y}, {f1.z, f1.w}, {f2.x, f2.y}};
+    const float2 el[3] = {{f2.z, f2.w}, {f3.x, f3.y}, {f3.z, f3.w}};
+    const float v0[3] = {f0.x, f0.y, f0.z};
+    const float nh[3] = {f4.x, f4.y, f4.z}, nl[3] = {f4.w, f5.x, f5.y};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        y.v0[c] = fr[c];
-        const ff e1 = {fr[o_e1h + c], fr[o_e1l + c]}, e2 = {fr[o_e2h + c], fr[o_e2l + c]};
-        y.n[c] = {fr[o_nh + c], fr[o_nl + c]};
-        y.p[c] = ff_add(ff_mul(e1, b1), ff_mul(e2, b2));
+        y.v0[c] = v0[c];
+        y.n[c] = {nh[c], nl[c]};
+        const ff2 t = ff_mul2(eh[c], el[c], b);  // (e1 b1, e2 b2)
+        const ff s = two_sum(t.hi.x, t.hi.y);
+        y.p[c] = fast_two_sum(s.hi, rn_sub(s.lo, rn_add(t.nlo.x, t.nlo.y)));
     }
+}
+
+// r = y - x of two points, component by component the float-float sum of the
+// exact difference of their first vertices and the difference of their offsets.
+__device__ __forceinline__ void point_diff(const FFPoint& y, const FFPoint& x, ff (&r)[3])
+{
+    const ff2 v = two_diff2(make_float2(y.v0[0], y.v0[1]), make_float2(x.v0[0], x.v0[1]));
+    ff2 d = two_diff2(make_float2(y.p[0].hi, y.p[1].hi), make_float2(x.p[0].hi, x.p[1].hi));
+    const float2 l = sub2(make_float2(y.p[0].lo, y.p[1].lo), make_float2(x.p[0].lo, x.p[1].lo));
+    d = fast_two_sub2(d.hi, sub2(d.nlo, l));
+    const ff2 s = two_sum2(v.hi, d.hi);
+    d = fast_two_sub2(s.hi, __fadd2_rn(s.nlo, __fadd2_rn(v.nlo, d.nlo)));
+    r[0] = {d.hi.x, -d.nlo.x};
+    r[1] = {d.hi.y, -d.nlo.y};
+    r[2] = ff_add(two_sum(y.v0[2], -x.v0[2]), ff_sub(y.p[2], x.p[2]));
 }
 
 __device__ __forceinline__ int64_t area_sample_ff(const WalkParams& p, StreamKey key, uint32_t q,
@@ -482,9 +538,7 @@ __global__ void __launch_bounds__(128, WOB_SL_MIN_BLOCKS) k_sl_walks_ff(WalkPara
                 } else {
                     j = area_sample_ff(p, key, q, w, (uint32_t)k, y, b0, b1f, b2f);
                     ff r[3];
-#pragma unroll
-                    for (int c = 0; c < 3; ++c)
-                        r[c] = ff_add(two_sum(y.v0[c], -x.v0[c]), ff_sub(y.p[c], x.p[c]));
+                    point_diff(y, x, r);
                     const float r2 =
                         __fmaf_rn(r[0].hi, r[0].hi, __fmaf_rn(r[1].hi, r[1].hi, r[2].hi * r[2].hi));
                     if (r2 < rmin2) break;  // empty sample
@@ -569,11 +623,9 @@ __device__ __forceinline__ ff ris_kernel(int bx, const FFPoint& x, const FFPoint
                                          float alpha, bool& close)
 {
     ff r[3];
+    point_diff(y, x, r);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        r[c] = ff_add(two_sum(y.v0[c], -x.v0[c]), ff_sub(y.p[c], x.p[c]));
-        r[c] = {rn_mul(r[c].hi, scale), rn_mul(r[c].lo, scale)};
-    }
+    for (int c = 0; c < 3; ++c) r[c] = {rn_mul(r[c].hi, scale), rn_mul(r[c].lo, scale)};
     const ff rr = ff_dot3(r, r);
     close = rr.hi < kRisClose2;
     // every condition's lanes together: alpha is 0 but on Robin parts

@@ -45,11 +45,9 @@ struct alignas(32) NormalArea {
 // value, the edges e1 = v1 - v0 and e2 = v2 - v0 (exact: differences of FP32
 // coordinates) and the unit normal; 96 bytes, read as six float4.
 struct alignas(16) TriFrame {
-    float v0[3];
-    float e1h[3], e1l[3];
-    float e2h[3], e2l[3];
-    float nh[3], nl[3];
-    float pad[3];
+    float v0[3], pad0;
+    float eh[3][2], el[3][2];  // edges e1, e2 side by side, hi and lo parts
+    float nh[3], nl[3], pad[2];
 };
 static_assert(sizeof(TriFrame) == 96, "six float4");
 
