@@ -347,8 +347,8 @@ __device__ __forceinline__ float fine_tri(const CvGeom& c, int j, float3 x, floa
 // rounded as the scalar operations round it, nodes 0, 2, 4 and 1, 3, 5 in two
 // sums that meet before node 6.  VALUE: fx counts (else 0, and S0 is not formed).
 // Bounded by the FMA pipe: 80 packed operations (two cycles each) for 63
-// instructions a triangle, 3.6 of the 9.5 -> 7.46 ms that the residual walks of
-// 8,192 queries x 64 walks x 2 vertices take (fine nodes 2.6).  A form with the
+// instructions a triangle: 3.6 of the 7.15 ms (9.5 before) that the residual walks
+// of 8,192 queries x 64 walks x 2 vertices take, the fine nodes 2.3.  A form with the
 // centroid's distance and offsets along two medians needs 30% fewer operations,
 // and rounds differently.
 template <bool VALUE>
@@ -577,6 +577,32 @@ __global__ void __launch_bounds__(kQuadThreads, 8) k_cv_quad_H(CvGeom c, int phi
 }
 
 // ------------------------------------------------------------ residual walks
+// A bucket: the part of a triangle (original id) a vertex lies on, its corner
+// sub-triangles or the middle one, kSubLevels times over.
+constexpr int kSubLevels = 1, kSubs = 1 << (2 * kSubLevels);
+
+__device__ __forceinline__ int sub_triangle(const float4* __restrict__ tv, int pos, float3 y)
+{
+    const float4 a = __ldg(tv + 3 * pos), b = __ldg(tv + 3 * pos + 1), c = __ldg(tv + 3 * pos + 2);
+    const float3 e1 = make_float3(b.x - a.x, b.y - a.y, b.z - a.z),
+                 e2 = make_float3(c.x - a.x, c.y - a.y, c.z - a.z),
+                 d = make_float3(y.x - a.x, y.y - a.y, y.z - a.z);
+    auto dot = [](float3 u, float3 v) { return u.x * v.x + u.y * v.y + u.z * v.z; };
+    const float g11 = dot(e1, e1), g12 = dot(e1, e2), g22 = dot(e2, e2), h1 = dot(d, e1), h2 = dot(d, e2);
+    const float inv = __fdividef(1.f, g11 * g22 - g12 * g12);
+    float b1 = (g22 * h1 - g12 * h2) * inv, b2 = (g11 * h2 - g12 * h1) * inv, b0 = 1.f - b1 - b2;
+    int id = 0;
+    for (int l = 0; l < kSubLevels; ++l) {  // any rounding is fine: a bucket is only an order
+        const int s = b0 > 0.5f ? 0 : b1 > 0.5f ? 1 : b2 > 0.5f ? 2 : 3;
+        const float k = s == 3 ? -2.f : 2.f, o = s == 3 ? 1.f : 0.f;
+        b0 = k * b0 + o - (s == 0);
+        b1 = k * b1 + o - (s == 1);
+        b2 = k * b2 + o - (s == 2);
+        id = 4 * id + s;
+    }
+    return id;
+}
+
 struct CvWalk {
     double* x;    // 3 x W
     double* S;    // walk sums = per-walk values
@@ -585,9 +611,9 @@ struct CvWalk {
     int* alive;   // 0 once a line missed
     float* vpos;  // 3 x W (contiguous per walk: x, y, z) for the network
     float* nut;   // network value at the current vertex
-    int* own;     // triangle of the current vertex (original id; T once dead)
-    int* perm;    // walks bucketed by `own` (the order k_cvw_accum visits them)
-    int* count;   // T + 1 bucket sizes
+    int* own;     // bucket of the current vertex (the last one, kSubs T, once dead)
+    int* perm;    // walks by bucket (the order k_cvw_accum visits them)
+    int* count;   // kSubs T + 1 bucket sizes
     int* incl;    // their inclusive prefix sums
     int* cursor;  // scatter cursors
     int64_t W;
@@ -606,7 +632,7 @@ __global__ void k_cvw_init(WalkParams p, CvWalk st)
         st.P[i] = 1.0;
         st.self[i] = -1;
         st.alive[i] = 1;
-        st.own[i] = st.T;
+        st.own[i] = kSubs * st.T;
         st.vpos[3 * i] = p.queries[3 * qi];
         st.vpos[3 * i + 1] = p.queries[3 * qi + 1];
         st.vpos[3 * i + 2] = p.queries[3 * qi + 2];
@@ -643,7 +669,7 @@ __global__ void __launch_bounds__(128, 4) k_cvw_trace(WalkParams p, CvWalk st, i
                                  err, p.iter_limit);
         if (t.m == 0) {
             st.alive[i] = 0;
-            st.own[i] = st.T;
+            st.own[i] = kSubs * st.T;
             continue;
         }
         const int pos = select_hit(p.tv, t, hits, key, q, w, (uint32_t)k);
@@ -658,14 +684,19 @@ __global__ void __launch_bounds__(128, 4) k_cvw_trace(WalkParams p, CvWalk st, i
         st.vpos[3 * i + 1] = y[1].hi;
         st.vpos[3 * i + 2] = y[2].hi;
         st.self[i] = pos;
-        st.own[i] = (int)prim_of(p.tv, pos);
+        st.own[i] = kSubs * (int)prim_of(p.tv, pos) +
+                    sub_triangle(p.tv, pos, make_float3(y[0].hi, y[1].hi, y[2].hi));
     }
     if (err) atomicOr(p.error_word, err);
 }
 
-// Bucket the walks by the triangle their vertex lies on (a counting sort;
-// dead walks go to bucket T, last).  Walks of one bucket share the near-field
-// candidate list, so a warp of them reads the same fine nodes.
+// Bucket the walks by the triangle their vertex lies on, and the part of it (a
+// counting sort; dead walks go to the last bucket).  Walks of one triangle share
+// the near-field candidate list, so a warp of them reads the same fine nodes;
+// walks of one part of it are near to nearly the same of them, so a warp sums
+// fewer that only some of its lanes need (524,288 walks on 1,280 triangles, two
+// vertices: 7.46 ms with whole triangles, 7.15 with four parts, 7.08 with
+// sixteen, whose counts would take 200 MB on the largest mesh).
 __global__ void k_cvw_count(CvWalk st)
 {
     // warp-uniform loop: every lane takes part in the match
@@ -681,7 +712,7 @@ __global__ void k_cvw_count(CvWalk st)
 
 __global__ void k_cvw_cursor(CvWalk st)
 {
-    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b <= st.T; b += gridDim.x * blockDim.x)
+    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b <= kSubs * st.T; b += gridDim.x * blockDim.x)
         st.cursor[b] = st.incl[b] - st.count[b];
 }
 
@@ -703,7 +734,7 @@ __global__ void __launch_bounds__(kQuadThreads, 8) k_cvw_accum(WalkParams p, CvW
 {
     __shared__ FarTile sm;
     const double phi = (double)p.phi;
-    const int64_t n_alive = st.T > 0 ? st.incl[st.T - 1] : 0;  // buckets 0..T-1
+    const int64_t n_alive = st.T > 0 ? st.incl[kSubs * st.T - 1] : 0;  // all but the last
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n_alive;
          base += (int64_t)gridDim.x * blockDim.x) {
         const bool ok = base + threadIdx.x < n_alive;
@@ -1085,7 +1116,7 @@ int wob_cv_solve(const wob_problem* prob, wob_cv c, const float* params, const f
     st.W = Q * (int64_t)walks;
     st.T = c->T;
     const size_t W = (size_t)st.W;
-    const size_t nb = (size_t)c->T + 1;
+    const size_t nb = (size_t)kSubs * c->T + 1;
     char* buf = nullptr;
     const size_t bytes = W * (8 * 5 + 4 * 2 + 4 * 4 + 4 * 2) + nb * 12 + 256;
     WOB_CUDA_TRY(cudaMallocAsync((void**)&buf, bytes, s));
