@@ -51,10 +51,9 @@ constexpr int64_t kGroupWalksPerSm = 200;
 #ifndef WOB_SL_MIN_BLOCKS
 #define WOB_SL_MIN_BLOCKS 7
 #endif
-// Resampled single-layer walks: 7 blocks of 128 threads per SM (72 registers).  On
-// 1.05e6 walks of the mixed torus 6 blocks took 1.61 ms, 7 1.52, 8 (64 registers)
-// 1.54.
-constexpr int kRisBlocks = 7;
+// Resampled single-layer walks: 6 blocks of 128 threads per SM (76 registers, no
+// spills; 7 blocks spill 72 bytes without and 16 with the sums in shared memory).
+constexpr int kRisBlocks = 6, kRisThreads = 128;
 
 // Tiles of 32 consecutive walks of one problem from its global counter
 // (dynamic balance), the 64-bit bookkeeping of the two tiles under way and
@@ -596,7 +595,7 @@ __global__ void __launch_bounds__(128, WOB_SL_MIN_BLOCKS) k_sl_walks_ff(WalkPara
 // the walk's weights, terms and sums FP64.  What bounds it is issue: some 400
 // FP32 instructions a candidate, where about 60 FP64 instructions, each worth
 // 64 FP32 issue slots on this GPU, took 14.1 ms for 1.05e6 walks x 4 vertices x 16
-// candidates (200,000 triangles).  Now 1.52 ms; 2.5 ms while lanes that stayed
+// candidates (200,000 triangles).  Now 1.48 ms; 2.5 ms while lanes that stayed
 // or had another condition branched apart (16 of 32 active).
 // ---------------------------------------------------------------------------
 
@@ -692,17 +691,26 @@ __device__ __forceinline__ double ris_data(const WalkParams& p, int64_t j, const
 }
 
 template <bool DEBUG>
-__global__ void __launch_bounds__(128, kRisBlocks) k_sl_walks_ris(WalkParams p)
+__global__ void __launch_bounds__(kRisThreads, kRisBlocks) k_sl_walks_ris(WalkParams p)
 {
     const StreamKey key{p.key0, p.key1};
     const int64_t total = p.Q * (int64_t)p.N;
     const double phi = (double)p.phi;
     const int se = ilogb(p.L);
     const float scale = scalbnf(1.f, -se), alpha = p.alpha / scale;
-    // |Gamma| / ris times the constant factors of K and the units' powers
-    const double wq = p.area / (double)p.ris / kFourPi * (double)scale;       // G
-    const double wd = wq * ((double)p.kmix / (double)p.pk);                   // (k / p_k) G
-    const double wl = 2.0 * wq * (double)scale;                               // 2 dG/dn_x
+    // |Gamma| / ris times the constant factors of K and the units' powers, and each
+    // walk's sums: in shared memory, off the candidates' registers (76 of them hold
+    // the loop without spills)
+    enum { kQueryW, kDirichletW, kLayerW };
+    enum { kSum, kProduct, kFirst };
+    __shared__ double weight[3], walk[3][kRisThreads];
+    if (threadIdx.x == 0) {
+        const double wq = p.area / (double)p.ris / kFourPi * (double)scale;  // G
+        weight[kQueryW] = wq;
+        weight[kDirichletW] = wq * ((double)p.kmix / (double)p.pk);          // (k / p_k) G
+        weight[kLayerW] = 2.0 * wq * (double)scale;                          // 2 dG/dn_x
+    }
+    __syncthreads();
     const int uniform_bc = p.kind == WOB_ROBIN_SL ? WOB_BC_ROBIN : WOB_BC_NEUMANN;
     ff wc[kMaxRis];
     const int lane = threadIdx.x & 31;
@@ -723,9 +731,10 @@ __global__ void __launch_bounds__(128, kRisBlocks) k_sl_walks_ris(WalkParams p)
             x.n[c] = {0.f, 0.f};
         }
         int bx = -1;
-        int64_t jx = -1;
+        int32_t jx = -1;
         float ux = 0.f, u2x = 0.f;
-        double S = 0.0, P = 1.0, W0 = 0.0;
+        walk[kSum][threadIdx.x] = walk[kFirst][threadIdx.x] = 0.0;
+        walk[kProduct][threadIdx.x] = 1.0;
         bool going = live;
         // every lane takes part in every step: a walk that stays, or has ended,
         // draws its candidates too and drops them (the warp would wait for the
@@ -783,23 +792,23 @@ __global__ void __launch_bounds__(128, kRisBlocks) k_sl_walks_ris(WalkParams p)
                     // parts, negative on Dirichlet parts (and for a zero kernel)
                     const float sg = bx < 0 ? wc[pick].hi : bx == WOB_BC_DIRICHLET ? -1.f
                                                           : -(float)p.phi * wc[pick].hi;
-                    const double wk = bx < 0 ? wq : bx == WOB_BC_DIRICHLET ? wd : wl;
+                    const double wk = weight[bx < 0 ? kQueryW : bx == WOB_BC_DIRICHLET ? kDirichletW : kLayerW];
                     wfac = (sg > 0.f ? wk : -wk) * ff_join(sumw);
                     x = y;
-                    jx = j;
+                    jx = (int32_t)j;
                     ux = u24f(u.z);
                     u2x = u24f(u.w);
                 }
-                if (k == 0) W0 = wfac; else P *= wfac;
+                if (k == 0) walk[kFirst][threadIdx.x] = wfac; else walk[kProduct][threadIdx.x] *= wfac;
                 const int by = p.bc_type ? (int)__ldg(p.bc_type + jx) : uniform_bc;
                 const double dat = ris_data(p, jx, x, ux, u2x, by);
                 double src = by == WOB_BC_DIRICHLET ? (double)p.kmix * dat : 2.0 * phi * dat;
                 if (k == p.M - 1) src *= 0.5;
-                S = fma(P, src, S);
+                walk[kSum][threadIdx.x] = fma(walk[kProduct][threadIdx.x], src, walk[kSum][threadIdx.x]);
                 bx = by;
             }
         }
-        const double value = W0 * S;
+        const double value = walk[kFirst][threadIdx.x] * walk[kSum][threadIdx.x];
         if (live) {
             if (p.per_walk) p.per_walk[idx] = value;
             if (DEBUG && p.walk_flag) p.walk_flag[idx] = 0;
@@ -1489,6 +1498,7 @@ int launch_dl_walks(const WalkParams& p, bool counted, bool debug, cudaStream_t 
 int launch_sl_walks(const WalkParams& p, bool debug, cudaStream_t s)
 {
     const int threads = 128;
+    static_assert(kRisThreads == threads, "one block size");
     const int64_t work = p.Q * (int64_t)p.N;
     if (p.ris > 1) {
         if (debug)
