@@ -51,9 +51,10 @@ constexpr int64_t kGroupWalksPerSm = 200;
 #ifndef WOB_SL_MIN_BLOCKS
 #define WOB_SL_MIN_BLOCKS 7
 #endif
-// Resampled single-layer walks: 6 blocks of 128 threads per SM (76 registers, no
-// spills; 7 blocks spill 72 bytes without and 16 with the sums in shared memory).
-constexpr int kRisBlocks = 6, kRisThreads = 128;
+// Resampled single-layer walks: 7 blocks of 128 threads per SM (71 registers, no
+// spills with the walk's sums and n_x in shared memory; 1.42 ms for 1.05e6 walks of
+// the mixed torus, 6 blocks with n_x in registers 1.48).
+constexpr int kRisBlocks = 7, kRisThreads = 128;
 
 // Tiles of 32 consecutive walks of one problem from its global counter
 // (dynamic balance), the 64-bit bookkeeping of the two tiles under way and
@@ -321,7 +322,7 @@ __device__ __forceinline__ int64_t area_pick(const WalkParams& p, uint32_t hi, u
 // rounded as ff.cuh's operations round it.  The low parts are kept negated (an
 // exact change): the packed operations take no negated operands, and the errors
 // come out of fma(a, -b, ab) and of differences without extra instructions.
-// Resampled walks 1.52 -> 1.38 ms against the scalar form (1.05e6 walks x 4
+// Resampled walks 1.52 -> 1.37 ms against the scalar form (1.05e6 walks x 4
 // vertices x 16 candidates), single-layer walks, which wait for their loads
 // rather than for issue, 4.53 -> 4.51 ms.
 struct ff2 {
@@ -592,11 +593,11 @@ __global__ void __launch_bounds__(128, WOB_SL_MIN_BLOCKS) k_sl_walks_ff(WalkPara
 // sources as in k_sl_walks_ff.  The pick compares running sums of |K|, so a
 // rounding can move it to another candidate: points, kernels and sums are
 // float-float (44 bits and more; a pick moves about once in 10^11 draws), and
-// the walk's weights, terms and sums FP64.  What bounds it is issue: some 400
-// FP32 instructions a candidate, where about 60 FP64 instructions, each worth
-// 64 FP32 issue slots on this GPU, took 14.1 ms for 1.05e6 walks x 4 vertices x 16
-// candidates (200,000 triangles).  Now 1.48 ms; 2.5 ms while lanes that stayed
-// or had another condition branched apart (16 of 32 active).
+// the walk's weights, terms and sums FP64.  What bounds it: a candidate's guide,
+// CDF and frame reads (L1 80% busy) and some 500 instructions, where about 60 FP64
+// instructions, each worth 64 FP32 issue slots on this GPU, took 14.1 ms for 1.05e6
+// walks x 4 vertices x 16 candidates (200,000 triangles).  Now 1.42 ms; 2.5 ms while
+// lanes that stayed or had another condition branched apart (16 of 32 active).
 // ---------------------------------------------------------------------------
 
 // 1 / sqrt(a) for a normal a: the fast root y, corrected to second order in
@@ -699,11 +700,12 @@ __global__ void __launch_bounds__(kRisThreads, kRisBlocks) k_sl_walks_ris(WalkPa
     const int se = ilogb(p.L);
     const float scale = scalbnf(1.f, -se), alpha = p.alpha / scale;
     // |Gamma| / ris times the constant factors of K and the units' powers, and each
-    // walk's sums: in shared memory, off the candidates' registers (76 of them hold
-    // the loop without spills)
+    // walk's sums and normal: in shared memory, off the candidates' registers (71 of
+    // them hold the loop without spills)
     enum { kQueryW, kDirichletW, kLayerW };
     enum { kSum, kProduct, kFirst };
     __shared__ double weight[3], walk[3][kRisThreads];
+    __shared__ volatile float normal[6][kRisThreads];  // n_x
     if (threadIdx.x == 0) {
         const double wq = p.area / (double)p.ris / kFourPi * (double)scale;  // G
         weight[kQueryW] = wq;
@@ -729,6 +731,7 @@ __global__ void __launch_bounds__(kRisThreads, kRisBlocks) k_sl_walks_ris(WalkPa
             x.v0[c] = p.queries[3 * qi + c];
             x.p[c] = {0.f, 0.f};
             x.n[c] = {0.f, 0.f};
+            normal[2 * c][threadIdx.x] = normal[2 * c + 1][threadIdx.x] = 0.f;
         }
         int bx = -1;
         int32_t jx = -1;
@@ -755,6 +758,9 @@ __global__ void __launch_bounds__(kRisThreads, kRisBlocks) k_sl_walks_ris(WalkPa
                 __syncwarp();  // the searches differ in length
                 frame_point_ff(p, j, u.z, u.w, y, b0, b1, b2);
                 bool close;
+#pragma unroll
+                for (int d = 0; d < 3; ++d)
+                    x.n[d] = {normal[2 * d][threadIdx.x], normal[2 * d + 1][threadIdx.x]};
                 ff K = ris_kernel(bx, x, y, scale, alpha, close);
                 if (close && going && !stay)
                     K = ris_kernel_close(p, bx, jx, make_float2(ux, u2x), p.queries + 3 * qi, j,
@@ -795,12 +801,20 @@ __global__ void __launch_bounds__(kRisThreads, kRisBlocks) k_sl_walks_ris(WalkPa
                     const double wk = weight[bx < 0 ? kQueryW : bx == WOB_BC_DIRICHLET ? kDirichletW : kLayerW];
                     wfac = (sg > 0.f ? wk : -wk) * ff_join(sumw);
                     x = y;
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        normal[2 * d][threadIdx.x] = y.n[d].hi;
+                        normal[2 * d + 1][threadIdx.x] = y.n[d].lo;
+                    }
                     jx = (int32_t)j;
                     ux = u24f(u.z);
                     u2x = u24f(u.w);
                 }
                 if (k == 0) walk[kFirst][threadIdx.x] = wfac; else walk[kProduct][threadIdx.x] *= wfac;
                 const int by = p.bc_type ? (int)__ldg(p.bc_type + jx) : uniform_bc;
+#pragma unroll
+                for (int d = 0; d < 3; ++d)
+                    x.n[d] = {normal[2 * d][threadIdx.x], normal[2 * d + 1][threadIdx.x]};
                 const double dat = ris_data(p, jx, x, ux, u2x, by);
                 double src = by == WOB_BC_DIRICHLET ? (double)p.kmix * dat : 2.0 * phi * dat;
                 if (k == p.M - 1) src *= 0.5;
