@@ -43,6 +43,7 @@
 // 41.9 ms.
 #pragma once
 
+#include "node_stack.cuh"
 #include "wob_device.cuh"
 
 namespace wob {
@@ -470,7 +471,7 @@ __device__ __forceinline__ void run_line_groups(P& pol, GroupShared& sm, int* st
                     for (int i = 0; i < 8 / kG; ++i)
                         hitm |= ((__ballot_sync(kAllLanes, (mine >> i) & 1u) >> gsh) & kGroupMask) << (kG * i);
                     if (trav) {
-                        uint32_t im = hitm & ((1u << nint) - 1u);
+                        const uint32_t im = hitm & ((1u << nint) - 1u);
                         const uint32_t lm = hitm ^ im;
                         if (lm) {
 #pragma unroll
@@ -482,25 +483,8 @@ __device__ __forceinline__ void run_line_groups(P& pol, GroupShared& sm, int* st
                             }
                             nq += __popc(lm);
                         }
-                        if (!im && sp > 0) {
-                            const uint32_t e = (uint32_t)mem.stack[--sp * kGroups];
-                            base = (int)(e & 0xFFFFFFu);
-                            im = e >> 24;
-                        }
-                        if (im) {
-                            node = base + __ffs(im) - 1;
-                            im &= im - 1;
-                            if (im) {
-                                if (sp < levels) {
-                                    if (j == 0) mem.stack[sp * kGroups] = base | (int)(im << 24);
-                                    ++sp;
-                                } else {
-                                    err |= 1;
-                                }
-                            }
-                        } else {
-                            trav = false;
-                        }
+                        trav = next_node(mem.stack, kGroups, levels, j == 0, base, im, sp, node, err,
+                                         [&] { __syncwarp(kGroupMask << gsh); });
                     }
                     __syncwarp();
                 }
