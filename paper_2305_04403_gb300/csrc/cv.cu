@@ -34,14 +34,31 @@ constexpr int kCoarse = 7;
 constexpr int kMaxFine = 7 * 64;  // level <= 3
 constexpr float kInvFourPi = 0.0795774715459476678f;
 
-__constant__ float c_coarse_b[kCoarse * 3];
-__constant__ float c_coarse_w[kCoarse];
-__constant__ float c_fine_b[kMaxFine * 3];
-__constant__ float c_fine_w[kMaxFine];
+// Radon's rule (degree 5): barycentric coordinates and weights of its seven
+// nodes, the centroid and two orbits of three.
+constexpr double kSqrt15 = 3.8729833462074168852;
+constexpr double kA1 = (6.0 - kSqrt15) / 21.0, kB1 = (9.0 + 2.0 * kSqrt15) / 21.0;
+constexpr double kA2 = (6.0 + kSqrt15) / 21.0, kB2 = (9.0 - 2.0 * kSqrt15) / 21.0;
+constexpr double kRule[kCoarse][3] = {{1.0 / 3, 1.0 / 3, 1.0 / 3}, {kB1, kA1, kA1}, {kA1, kB1, kA1},
+                                      {kA1, kA1, kB1}, {kB2, kA2, kA2}, {kA2, kB2, kA2}, {kA2, kA2, kB2}};
+constexpr float kW0 = (float)(9.0 / 40.0), kW1 = (float)((155.0 - kSqrt15) / 1200.0),
+                kW2 = (float)((155.0 + kSqrt15) / 1200.0);
+
+// The same in every object, at every level (a fine node's weight is the rule's
+// times 4^-level, exact: CvGeom::sub_w): nothing here is written after the
+// module is loaded, so objects of several levels and streams live side by side.
+#define WOB_RULE_ROW(q) (float)kRule[q][0], (float)kRule[q][1], (float)kRule[q][2]
+__constant__ float c_coarse_b[kCoarse * 3] = {WOB_RULE_ROW(0), WOB_RULE_ROW(1), WOB_RULE_ROW(2),
+                                              WOB_RULE_ROW(3), WOB_RULE_ROW(4), WOB_RULE_ROW(5),
+                                              WOB_RULE_ROW(6)};
+#undef WOB_RULE_ROW
+__constant__ float c_orbit_w[3] = {kW0, kW1, kW2};
+__constant__ float c_coarse_w[kCoarse] = {kW0, kW1, kW1, kW1, kW2, kW2, kW2};
 
 struct CvGeom {
     int T;
     int F;                       // fine nodes per triangle
+    float sub_w;                 // a sub-triangle's share of its triangle, 4^-level
     const float4* tri_c;         // centroid, near radius (near x longest edge)
     const float4* tri_p;         // unit normal n, plane offset n . y of the triangle
     const float* tri_a;          // area
@@ -51,24 +68,10 @@ struct CvGeom {
     const int* cand;
 };
 
-// Radon's rule (degree 5) in barycentric coordinates and its
-// 4^level-subdivided version, computed once in double.
-void rule_tables(int level, std::vector<float>& cb, std::vector<float>& cw,
-                 std::vector<float>& fb, std::vector<float>& fw)
+// Barycentric coordinates of the fine nodes: the rule on each of a triangle's
+// 4^level sub-triangles, computed in double.
+std::vector<float> fine_rule(int level)
 {
-    const double s15 = std::sqrt(15.0);
-    const double a1 = (6.0 - s15) / 21.0, b1 = (9.0 + 2.0 * s15) / 21.0;
-    const double a2 = (6.0 + s15) / 21.0, b2 = (9.0 - 2.0 * s15) / 21.0;
-    const double w1 = (155.0 - s15) / 1200.0, w2 = (155.0 + s15) / 1200.0;
-    const double P[7][3] = {{1.0 / 3, 1.0 / 3, 1.0 / 3}, {b1, a1, a1}, {a1, b1, a1}, {a1, a1, b1},
-                            {b2, a2, a2}, {a2, b2, a2}, {a2, a2, b2}};
-    const double W[7] = {9.0 / 40.0, w1, w1, w1, w2, w2, w2};
-    cb.clear();
-    cw.clear();
-    for (int q = 0; q < 7; ++q) {
-        for (int c = 0; c < 3; ++c) cb.push_back((float)P[q][c]);
-        cw.push_back((float)W[q]);
-    }
     // sub-triangles as barycentric corner triples
     std::vector<std::array<std::array<double, 3>, 3>> tris;
     tris.push_back({{{1, 0, 0}, {0, 1, 0}, {0, 0, 1}}});
@@ -88,14 +91,12 @@ void rule_tables(int level, std::vector<float>& cb, std::vector<float>& cw,
         }
         tris = nxt;
     }
-    fb.clear();
-    fw.clear();
+    std::vector<float> fb;
     for (auto& T : tris)
-        for (int q = 0; q < 7; ++q) {
+        for (int q = 0; q < kCoarse; ++q)
             for (int c = 0; c < 3; ++c)
-                fb.push_back((float)(P[q][0] * T[0][c] + P[q][1] * T[1][c] + P[q][2] * T[2][c]));
-            fw.push_back((float)(W[q] / tris.size()));
-        }
+                fb.push_back((float)(kRule[q][0] * T[0][c] + kRule[q][1] * T[1][c] + kRule[q][2] * T[2][c]));
+    return fb;
 }
 
 // Far-field records: what the far field reads of a triangle, two triangles to
@@ -114,7 +115,8 @@ __device__ __forceinline__ float* far_slot(float4* far, int64_t j, int slot)
 }
 
 __global__ void k_cv_nodes(const float* __restrict__ verts, const int32_t* __restrict__ tris,
-                           int T, int F, float near, float4* __restrict__ tri_c,
+                           int T, int F, float near, const float* __restrict__ fine_b,
+                           float sub_w, float4* __restrict__ tri_c,
                            float4* __restrict__ tri_p, float* __restrict__ tri_R,
                            float* __restrict__ tri_a, float4* __restrict__ coarse,
                            float4* __restrict__ fine, float4* __restrict__ far)
@@ -168,10 +170,10 @@ __global__ void k_cv_nodes(const float* __restrict__ verts, const int32_t* __res
         for (int q = 0; q < F; ++q) {
             double p[3];
             for (int c = 0; c < 3; ++c)
-                p[c] = c_fine_b[3 * q] * v[0][c] + c_fine_b[3 * q + 1] * v[1][c] +
-                       c_fine_b[3 * q + 2] * v[2][c];
+                p[c] = fine_b[3 * q] * v[0][c] + fine_b[3 * q + 1] * v[1][c] +
+                       fine_b[3 * q + 2] * v[2][c];
             fine[(int64_t)F * j + q] = make_float4((float)p[0], (float)p[1], (float)p[2],
-                                                   (float)(c_fine_w[q] * area));
+                                                   (float)(c_coarse_w[q % kCoarse] * sub_w * area));
         }
     }
 }
@@ -310,21 +312,24 @@ __device__ __forceinline__ float fine_sum(const CvGeom& c, const float4* nd, int
                                           float fx, float sum)
 {
     const float4 tp = __ldg(c.tri_p + j);
-    const float area = __ldg(c.tri_a + j);
+    const float area = __ldg(c.tri_a + j) * c.sub_w;
     const NegPoint2 nx{make_float2(-x.x, -x.x), make_float2(-x.y, -x.y), make_float2(-x.z, -x.z)};
     float2 s1p = make_float2(0.f, 0.f), s0p = make_float2(0.f, 0.f);
     auto pair = [&](int q, float2 om) {
         node_acc2(SHARED ? nd[2 * q] : __ldg(nd + 2 * q), SHARED ? nd[2 * q + 1] : __ldg(nd + 2 * q + 1),
                   om, nx, s1p, s0p);
     };
+    // S0 with the rule's own weights; the fine nodes' 4^-level joins the area (a
+    // power of two: no rounding differs)
+    const float w0 = c_orbit_w[0], w1 = c_orbit_w[1], w2 = c_orbit_w[2];
     if (c.F == kCoarse) {  // level 0: one triangle, three pairs and the odd node
-#pragma unroll
-        for (int q = 0; q < kCoarse / 2; ++q) pair(q, make_float2(c_fine_w[2 * q], c_fine_w[2 * q + 1]));
+        pair(0, make_float2(w0, w1));
+        pair(1, make_float2(w1, w1));
+        pair(2, make_float2(w2, w2));
         float s1 = s1p.x + s1p.y, s0 = s0p.x + s0p.y;
-        node_acc(SHARED ? nd[c.F - 1] : __ldg(nd + c.F - 1), c_fine_w[kCoarse - 1], x, s1, s0);
+        node_acc(SHARED ? nd[c.F - 1] : __ldg(nd + c.F - 1), w2, x, s1, s0);
         return tri_term(tp, area, x, fx, s1, s0, sum);
     }
-    const float w0 = c_fine_w[0], w1 = c_fine_w[1], w2 = c_fine_w[4];  // centroid, orbits
     for (int g = 0; g < c.F; g += 2 * kCoarse, nd += 2 * kCoarse) {
         pair(0, make_float2(w0, w1));
         pair(1, make_float2(w1, w1));
@@ -908,9 +913,11 @@ struct wob_cv_s {
     float *tri_R = nullptr, *tri_a = nullptr, *coarse_val = nullptr, *fine_val = nullptr;
     int *cand_off = nullptr, *cand = nullptr;
     int64_t n_cand = 0;
+    // a sub-triangle's share of its triangle
+    float sub_w() const { return 1.f / (float)(1 << (2 * level)); }
     CvGeom geom() const
     {
-        return CvGeom{T, F, tri_c, tri_p, tri_a, far, fine_pk, cand_off, cand};
+        return CvGeom{T, F, sub_w(), tri_c, tri_p, tri_a, far, fine_pk, cand_off, cand};
     }
 };
 
@@ -968,8 +975,7 @@ int wob_cv_create(wob_mesh m, int32_t level, float near, void* stream, wob_cv* o
     c->level = level;
     c->near = near;
     c->F = 7 << (2 * level);
-    std::vector<float> cb, cw, fb, fw;
-    rule_tables(level, cb, cw, fb, fw);
+    const std::vector<float> rule = fine_rule(level);
     auto fail = [&](int code, const char* msg) {
         set_error("wob_cv_create: %s", msg);
         cudaStreamSynchronize(s);
@@ -977,11 +983,6 @@ int wob_cv_create(wob_mesh m, int32_t level, float near, void* stream, wob_cv* o
         delete c;
         return code;
     };
-    if (cudaMemcpyToSymbolAsync(c_coarse_b, cb.data(), cb.size() * 4, 0, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemcpyToSymbolAsync(c_coarse_w, cw.data(), cw.size() * 4, 0, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemcpyToSymbolAsync(c_fine_b, fb.data(), fb.size() * 4, 0, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemcpyToSymbolAsync(c_fine_w, fw.data(), fw.size() * 4, 0, cudaMemcpyHostToDevice, s) != cudaSuccess)
-        return fail(WOB_ERR_CUDA, "rule upload failed");
     const int T = c->T;
     if (cudaMalloc((void**)&c->tri_c, T * sizeof(float4)) != cudaSuccess ||
         cudaMalloc((void**)&c->tri_p, T * sizeof(float4)) != cudaSuccess ||
@@ -995,12 +996,17 @@ int wob_cv_create(wob_mesh m, int32_t level, float near, void* stream, wob_cv* o
         cudaMalloc((void**)&c->fine_val, (size_t)T * c->F * sizeof(float)) != cudaSuccess ||
         cudaMalloc((void**)&c->cand_off, T * sizeof(int)) != cudaSuccess)
         return fail(WOB_ERR_OOM, "device allocation failed");
+    // the barycentrics wait in fine_pk, which is written after the nodes are made
+    float* fine_b = (float*)c->fine_pk;
+    if (cudaMemcpyAsync(fine_b, rule.data(), rule.size() * sizeof(float), cudaMemcpyHostToDevice, s) != cudaSuccess)
+        return fail(WOB_ERR_CUDA, "rule upload failed");
     cudaMemsetAsync(c->coarse_val, 0, (size_t)T * kCoarse * sizeof(float), s);
     cudaMemsetAsync(c->fine_val, 0, (size_t)T * c->F * sizeof(float), s);
     const int threads = 128;
     const int grid = grid_for((const void*)k_cv_nodes, threads, 0, T);
-    k_cv_nodes<<<grid, threads, 0, s>>>(m->d.verts, m->d.tris, T, c->F, near, c->tri_c, c->tri_p,
-                                        c->tri_R, c->tri_a, c->coarse, c->fine, c->far);
+    k_cv_nodes<<<grid, threads, 0, s>>>(m->d.verts, m->d.tris, T, c->F, near, fine_b,
+                                        c->sub_w(), c->tri_c, c->tri_p, c->tri_R, c->tri_a,
+                                        c->coarse, c->fine, c->far);
     if (pack_nodes(c, s) != WOB_OK) return fail(WOB_ERR_CUDA, "node setup failed");
     int* count = nullptr;
     if (cudaMallocAsync((void**)&count, T * sizeof(int), s) != cudaSuccess)
