@@ -471,9 +471,17 @@ struct PointTile {
 };
 static_assert(sizeof(PointTile) <= 48 * 1024, "static shared memory");
 
+// A sum of near terms, s += v with the rounding error kept: a point may have
+// every triangle of the mesh near (any near > 0 is taken).
+__device__ __forceinline__ void add_near(ff& s, float v)
+{
+    const ff t = two_sum(s.hi, v);
+    s = {t.hi, s.lo + t.lo};
+}
+
 // The fine-node terms of `count` queued pairs, added to their lanes' sums.
 __device__ __forceinline__ void near_pairs(const CvGeom& c, const int* queue, int count, float3 x,
-                                           float& sum)
+                                           ff& sum)
 {
     const int lane = threadIdx.x & 31, sub = lane & (kPairLanes - 1), pairs = c.F >> 1;
     __syncwarp();
@@ -494,13 +502,13 @@ __device__ __forceinline__ void near_pairs(const CvGeom& c, const int* queue, in
         const float term = e < count ? tri_term(__ldg(c.tri_p + j), 0.f, y, 0.f, s1, 0.f, 0.f) : 0.f;
         for (int g = 0; g < 32; g += kPairLanes) {
             const float v = __shfl_sync(0xFFFFFFFFu, term, g);
-            if (lane == __shfl_sync(0xFFFFFFFFu, who, g)) sum += v;
+            if (lane == __shfl_sync(0xFFFFFFFFu, who, g)) add_near(sum, v);
         }
     }
     __syncwarp();
 }
 
-__global__ void __launch_bounds__(32 * kPointWarps) k_cv_quad_D(CvGeom c, const float* __restrict__ x,
+__global__ void __launch_bounds__(32 * kPointWarps, 4) k_cv_quad_D(CvGeom c, const float* __restrict__ x,
                                                                 int64_t n, float* out)
 {
     __shared__ PointTile sm;
@@ -515,7 +523,7 @@ __global__ void __launch_bounds__(32 * kPointWarps) k_cv_quad_D(CvGeom c, const 
                             : make_float3(0.f, 0.f, 0.f);
         const NegPoint2 nx{make_float2(-p.x, -p.x), make_float2(-p.y, -p.y), make_float2(-p.z, -p.z)};
         double tot = 0.0;
-        float near_tot = 0.f;
+        ff near_tot = {0.f, 0.f};
         int queued = 0;
         for (int j0 = 0; j0 < c.T; j0 += kPointTris) {
             const int recs = (min(kPointTris, c.T - j0) + 1) >> 1;
@@ -549,7 +557,7 @@ __global__ void __launch_bounds__(32 * kPointWarps) k_cv_quad_D(CvGeom c, const 
             tot += (double)part;
         }
         near_pairs(c, queue, queued, p, near_tot);
-        sm.sum[warp][lane] = tot + (double)near_tot;
+        sm.sum[warp][lane] = tot + ((double)near_tot.hi + (double)near_tot.lo);
         __syncthreads();
         if (warp == 0 && ok) {
             for (int k = 1; k < kPointWarps; ++k) tot = k == 1 ? sm.sum[0][lane] + sm.sum[1][lane] : tot + sm.sum[k][lane];
