@@ -46,16 +46,6 @@ int grid_for(const void* kernel, int threads, size_t smem, int64_t work_items)
     return (int)(need < full ? need : full);
 }
 
-int line_stack_bytes(const void* kernel, int entries, size_t& bytes)
-{
-    bytes = (size_t)entries * sizeof(int);
-    // above 48 KB in total (trees of more than about 50 levels) a kernel needs leave
-    if (bytes > 24 * 1024)
-        WOB_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)bytes));
-    return WOB_OK;
-}
-
 int check_problem(const wob_problem* prob)
 {
     if (!prob || !prob->bvh) {

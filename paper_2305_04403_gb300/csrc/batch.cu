@@ -316,20 +316,18 @@ const void* batch_kernel(int rounds)
            : rounds == 2 ? (const void*)k_batch_lines<2> : (const void*)k_batch_lines<1>;
 }
 
-// Grid and dynamic shared memory of a launch (sets the kernel's limit:
-// before any capture).
-int batch_grid(const wob_batch_s& b, int rounds, int64_t n_tiles, int& grid, size_t& smem)
+int batch_grid(const wob_batch_s& b, int rounds, int64_t n_tiles)
 {
-    WOB_TRY(line_stack_bytes(batch_kernel(rounds), b.levels * kLineThreads, smem));
-    grid = grid_for(batch_kernel(rounds), kLineThreads, smem, n_tiles * 32);
-    return WOB_OK;
+    return grid_for(batch_kernel(rounds), kLineThreads, line_stack_bytes(b.levels, kLineThreads),
+                    n_tiles * 32);
 }
 
 // Counter reset + walk kernel (no API call here may break stream capture).
 int launch_batch_kernels(wob_batch_s& b, const BatchProblem* probs, const Tile* tiles,
-                         int64_t n_tiles, int rounds, int grid, size_t smem, double* part,
-                         int64_t n_slots, cudaStream_t s)
+                         int64_t n_tiles, int rounds, int grid, double* part, int64_t n_slots,
+                         cudaStream_t s)
 {
+    const size_t smem = line_stack_bytes(b.levels, kLineThreads);
     WOB_CUDA_TRY(cudaMemsetAsync(b.counter, 0, sizeof(unsigned long long), s));
     WOB_CUDA_TRY(cudaMemsetAsync(b.err, 0, sizeof(int), s));  // this run's checks
     WOB_CUDA_TRY(cudaMemsetAsync(part, 0, n_slots * 2 * sizeof(double), s));  // added into
@@ -388,13 +386,11 @@ int autotune(wob_batch_s& b, const std::vector<double>& cost, cudaStream_t s)
             }
             cudaMemcpy(dt, t.data(), t.size() * sizeof(Tile), cudaMemcpyHostToDevice);
             float ms = 0.f, best_rep = 1e30f;
-            int grid = 1;
-            size_t smem = 0;
-            rc = batch_grid(b, rounds_c[ri], (int64_t)t.size(), grid, smem);
+            const int grid = batch_grid(b, rounds_c[ri], (int64_t)t.size());
             for (int rep = 0; rep < 2 && rc == WOB_OK; ++rep) {  // first run warms caches
                 cudaEventRecord(e0, s);
                 rc = launch_batch_kernels(b, dprobs, dt, (int64_t)t.size(), rounds_c[ri], grid,
-                                          smem, b.part, base, s);
+                                          b.part, base, s);
                 cudaEventRecord(e1, s);
                 cudaEventSynchronize(e1);
                 cudaEventElapsedTime(&ms, e0, e1);
@@ -566,13 +562,11 @@ int wob_batch_create(const wob_problem* problems, int32_t P, const int64_t* quer
         set_error("wob_batch_create: stream creation failed");
         return fail(WOB_ERR_CUDA);
     }
-    int g_walk = 1;
-    size_t smem = 0;
-    if ((rc = batch_grid(*b, b->rounds, b->n_tiles, g_walk, smem)) != WOB_OK) return fail(rc);
+    const int g_walk = batch_grid(*b, b->rounds, b->n_tiles);
     const int g_red = grid_for((const void*)k_reduce_batched, 256, 0, b->Qt * 32);
     cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal);
-    rc = launch_batch_kernels(*b, b->probs, b->tiles, b->n_tiles, b->rounds, g_walk, smem,
-                              b->part, b->n_slots, b->cap_stream);
+    rc = launch_batch_kernels(*b, b->probs, b->tiles, b->n_tiles, b->rounds, g_walk, b->part,
+                              b->n_slots, b->cap_stream);
     if (rc == WOB_OK && b->Qt > 0)
         k_reduce_batched<<<g_red, 256, 0, b->cap_stream>>>(b->part, b->qoff_dev,
                                                            b->part_base_dev, b->walks_dev, P,

@@ -109,6 +109,14 @@ struct LineShared {
     }
 };
 
+// Dynamic shared memory of a launch: a stack of one entry per level of the
+// tree for each of a block's `stacks`.  The deepest tree that is built (its binary
+// tree has fewer than kStackSize levels) stays within the 48 KB that every
+// kernel may use, so no launch changes a kernel's limit, which all threads share.
+inline size_t line_stack_bytes(int levels, int stacks) { return (size_t)levels * stacks * sizeof(int); }
+static_assert(sizeof(LineShared) + sizeof(int) * kStackSize * kLineThreads <= 48 * 1024,
+              "static shared memory and the deepest tree's stacks");
+
 // Header and quantised planes of a wide node, as two 32-byte loads (nodes are
 // 96 bytes from an allocation's start: 32-byte aligned).
 __device__ __forceinline__ void load_node(const float4* nd, float4& h, uint4& qx, uint4& qy, uint4& qz)

@@ -1467,8 +1467,7 @@ namespace {
 template <class K, class... Args>
 int launch_lines(K kernel, const WalkParams& p, cudaStream_t s, Args... args)
 {
-    size_t smem = 0;
-    WOB_TRY(line_stack_bytes((const void*)kernel, p.stack_levels * kLineThreads, smem));
+    const size_t smem = line_stack_bytes(p.stack_levels, kLineThreads);
     kernel<<<grid_for((const void*)kernel, kLineThreads, smem, p.Q * (int64_t)p.N), kLineThreads,
              smem, s>>>(p, args...);
     WOB_CUDA_TRY(cudaGetLastError());
@@ -1479,8 +1478,7 @@ int launch_lines(K kernel, const WalkParams& p, cudaStream_t s, Args... args)
 template <class K, class... Args>
 int launch_groups(K kernel, const WalkParams& p, cudaStream_t s, Args... args)
 {
-    size_t smem = 0;
-    WOB_TRY(line_stack_bytes((const void*)kernel, p.stack_levels * kGroups, smem));
+    const size_t smem = line_stack_bytes(p.stack_levels, kGroups);
     kernel<<<grid_for((const void*)kernel, kGroupThreads, smem, kG * p.Q * (int64_t)p.N),
              kGroupThreads, smem, s>>>(p, args...);
     WOB_CUDA_TRY(cudaGetLastError());

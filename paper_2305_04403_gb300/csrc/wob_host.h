@@ -39,10 +39,6 @@ void fill_params(WalkParams& p, const wob_problem* prob, const float* queries,
 // Persistent-grid size: SM count x resident blocks of `kernel` at `threads`.
 int grid_for(const void* kernel, int threads, size_t smem, int64_t work_items);
 
-// Bytes of dynamic shared memory for `entries` of the line engine's traversal
-// stacks, allowed for `kernel`.
-int line_stack_bytes(const void* kernel, int entries, size_t& bytes);
-
 // Arrays laid out one after another in a single allocation (256-byte aligned,
 // as cudaMalloc's): add() gives each array's offset, size() what to allocate.  A
 // mesh and its tree are two allocations instead of eleven; with those and their
