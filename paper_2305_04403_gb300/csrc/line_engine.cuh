@@ -110,10 +110,10 @@ struct LineShared {
 };
 
 // Dynamic shared memory of a launch: a stack of one entry per level of the
-// tree for each of a block's `stacks`.  The deepest tree that is built (its binary
+// tree for each of a block's `threads`.  The deepest tree that is built (its binary
 // tree has fewer than kStackSize levels) stays within the 48 KB that every
 // kernel may use, so no launch changes a kernel's limit, which all threads share.
-inline size_t line_stack_bytes(int levels, int stacks) { return (size_t)levels * stacks * sizeof(int); }
+inline size_t line_stack_bytes(int levels, int threads) { return (size_t)levels * threads * sizeof(int); }
 static_assert(sizeof(LineShared) + sizeof(int) * kStackSize * kLineThreads <= 48 * 1024,
               "static shared memory and the deepest tree's stacks");
 
@@ -416,6 +416,8 @@ struct GroupShared {
     int hits[kGroups][kMaxHits];
     unsigned long long tile;
 };
+static_assert(sizeof(GroupShared) + sizeof(int) * kStackSize * kGroupThreads <= 48 * 1024,
+              "static shared memory and the deepest tree's stacks");
 
 template <class P>
 __device__ __forceinline__ void run_line_groups(P& pol, GroupShared& sm, int* stack_base, int levels,
@@ -423,7 +425,8 @@ __device__ __forceinline__ void run_line_groups(P& pol, GroupShared& sm, int* st
 {
     const int lane = threadIdx.x & 31, j = lane & (kG - 1), gsh = lane & ~(kG - 1);
     const int grp = threadIdx.x / kG;  // the walk of the tile this lane works for
-    const GroupMem mem{sm.xd + grp, sm.acc + grp, sm.ids + grp, sm.lq + grp, stack_base + grp};
+    // (the stack is this lane's: next_node)
+    const GroupMem mem{sm.xd + grp, sm.acc + grp, sm.ids + grp, sm.lq + grp, stack_base + threadIdx.x};
     int* hits = sm.hits[grp];
     while (true) {
         int cnt = 0;
@@ -491,13 +494,14 @@ __device__ __forceinline__ void run_line_groups(P& pol, GroupShared& sm, int* st
                             }
                             nq += __popc(lm);
                         }
-                        trav = next_node(mem.stack, kGroups, levels, j == 0, base, im, sp, node, err,
-                                         [&] { __syncwarp(kGroupMask << gsh); });
+                        trav = next_node(mem.stack, kGroupThreads, levels, base, im, sp, node, err);
                     }
-                    __syncwarp();
                 }
+                __syncwarp();
                 // the queued leaves, kG at a time
-                const LineShear L = line_shear(o, d);
+                // (point and axis read again: six registers fewer in the node phase)
+                const LineShear L = line_shear(make_float3(mem.x_hi(0), mem.x_hi(1), mem.x_hi(2)),
+                                               make_float3(mem.d_hi(0), mem.d_hi(1), mem.d_hi(2)));
                 const float Tthr = g.edge_thr_L * fabsf(L.Sz);
                 for (int i0 = 0; __any_sync(kAllLanes, i0 < nq); i0 += kG) {
                     const bool have = i0 + j < nq;

@@ -1,6 +1,5 @@
-// node_stack.cuh -- the step from one wide node to the next of a line that a
-// group of lanes follows together, on one traversal stack for the group.
-// Compiles as plain C++ for the host tests.
+// node_stack.cuh -- the step of a line's traversal from one wide node to the
+// next.  Compiles as plain C++ for the host tests.
 #pragma once
 
 #include <cstdint>
@@ -13,35 +12,32 @@
 
 namespace wob {
 
-// base, im: first interior child of the node just tested and the mask of those
-// the line meets (the same in every lane of the group).  Takes the next node --
-// the first of these, or of the entry popped when there is none -- and pushes
-// the siblings that are left; false: the traversal is complete.  Every lane
-// reads the popped entry and the leader may write the same slot again in the
-// same turn, so sync() (a barrier of the group's lanes, ordering memory) stands
-// between the two: lanes that have branched apart need not be back together.
-// The caller has such a barrier before the next turn, whose lanes read what the
-// leader pushed here.
-template <class Sync>
-WOB_STACK_FN bool next_node(volatile int* stack, int stride, int levels, bool leader, int base,
-                            uint32_t im, int& sp, int& node, int& err, Sync sync)
+// base, mask: first interior child of the node just tested and those of them
+// that the line meets (base is a leaf's reference, below zero, in a node that has
+// no interior child, and counts only with a mask).  Takes the next node -- the
+// first of these, or of the entry popped when there is none -- and pushes the
+// siblings that are left; false: the traversal is complete.  The stack is the
+// calling lane's own, entry i at stack[i * stride]: lanes that follow one line
+// together each keep a copy, since within a turn nothing orders one lane's push
+// against another's pop.
+WOB_STACK_FN bool next_node(volatile int* stack, int stride, int levels, int base, uint32_t mask,
+                            int& sp, int& node, int& err)
 {
-    if (!im) {
-        if (sp == 0) return false;
+    if (!mask && sp > 0) {
         const uint32_t e = (uint32_t)stack[--sp * stride];
         base = (int)(e & 0xFFFFFFu);
-        im = e >> 24;
-        sync();
+        mask = e >> 24;
     }
+    if (!mask) return false;
 #if defined(__CUDA_ARCH__)
-    node = base + __ffs(im) - 1;
+    node = base + __ffs(mask) - 1;
 #else
-    node = base + __builtin_ctz(im);
+    node = base + __builtin_ctz(mask);
 #endif
-    im &= im - 1;
-    if (im) {
+    mask &= mask - 1;
+    if (mask) {
         if (sp < levels) {
-            if (leader) stack[sp * stride] = base | (int)(im << 24);
+            stack[sp * stride] = base | (int)(mask << 24);
             ++sp;
         } else {
             err |= 1;

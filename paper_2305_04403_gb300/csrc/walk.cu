@@ -1478,7 +1478,7 @@ int launch_lines(K kernel, const WalkParams& p, cudaStream_t s, Args... args)
 template <class K, class... Args>
 int launch_groups(K kernel, const WalkParams& p, cudaStream_t s, Args... args)
 {
-    const size_t smem = line_stack_bytes(p.stack_levels, kGroups);
+    const size_t smem = line_stack_bytes(p.stack_levels, kGroupThreads);
     kernel<<<grid_for((const void*)kernel, kGroupThreads, smem, kG * p.Q * (int64_t)p.N),
              kGroupThreads, smem, s>>>(p, args...);
     WOB_CUDA_TRY(cudaGetLastError());
