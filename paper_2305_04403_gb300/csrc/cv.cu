@@ -455,24 +455,34 @@ __device__ __forceinline__ float quad_sum(const CvGeom& c, FarTile& sm, float3 x
 }
 
 // (D f)(x0) at points off the surface: the quadrature of quad_sum with
-// f(x) = 0 and no own triangle.  A block takes 32 points, lane = point, and its
-// warps share the triangles (16 records each of a staged tile), so that a call
-// of few points still fills the SMs.  Points off the surface have no candidate
-// list and the 32 of a warp lie anywhere: their (point, near triangle) pairs
-// are queued, and eight lanes sum the fine nodes of one pair.  Evaluating a
-// triangle's fine nodes for the whole warp whenever it is near to one lane took
-// 1,196 us at 8,192 points and 1,280 triangles (18 near to each point), most of
-// it for lanes that did not need them; this form 66 us.
+// f(x) = 0 and no own triangle; lane = point, 32 points to a set.  The SPLIT warps
+// of a set share the triangles of a staged tile, so that a call of few points
+// still fills the SMs; with points enough for that, every warp has a set of its own
+// (SPLIT 1; launch_quad_D).  The far field is FP32 over runs of at most
+// kPointRun records, FP64 across them; the near triangles' terms add up in a
+// float-float pair.
+// Points off the surface have no candidate list and the 32 of a warp lie
+// anywhere.  A triangle near to few of them joins a queue of (point, triangle)
+// pairs, of which eight lanes sum the fine nodes of one; a triangle near to
+// enough of them is summed by every lane for its own point (all_near).
+// Evaluating each near triangle by every lane took 1,196 us at 8,192 points and
+// 1,280 triangles (18 near to each point), most of it for lanes that did not need
+// it, the queue 66 us; with all 20 triangles of a coarse boundary near to 100,000
+// points the queue took 368 us, the form before it 23 and this one 21 (level 0).
 constexpr int kPointWarps = 8, kPointTris = 256, kPairQueue = 128, kPairLanes = 8;
+constexpr int kPointRun = kPointTris / 2 / kPointWarps;
+constexpr int kPairStage = 16;  // pairs of nodes that a warp stages for all its lanes
 struct PointTile {
     float4 rec[kPointTris / 2 * kFarRec];
     int queue[kPointWarps][kPairQueue];  // lane << 20 | triangle
-    double sum[kPointWarps][32];
+    union {
+        float4 fine[kPointWarps][2 * kPairStage];
+        double sum[kPointWarps][32];
+    };
 };
 static_assert(sizeof(PointTile) <= 48 * 1024, "static shared memory");
 
-// A sum of near terms, s += v with the rounding error kept: a point may have
-// every triangle of the mesh near (any near > 0 is taken).
+// A sum of near terms, s += v with the rounding error kept.
 __device__ __forceinline__ void add_near(ff& s, float v)
 {
     const ff t = two_sum(s.hi, v);
@@ -508,16 +518,78 @@ __device__ __forceinline__ void near_pairs(const CvGeom& c, const int* queue, in
     __syncwarp();
 }
 
+// Whether a triangle near to `lanes` points of a warp is summed by every lane: its
+// F / 2 pairs of nodes for the warp, against F / 64 pairs and a fixed cost (the
+// shuffles, as 2 pairs) for each point in the queue, whose loads are the slower
+// ones.  Over 534 calls (20 to 1,280 triangles, every level, near 0.5 to 8, points
+// inside and close to the surface) the line at 20 F took 0.336 of the time of the
+// lane-per-point form before the queue; at 32 F 0.345, with 64 for 128 0.343 to 0.347.
+__device__ __forceinline__ bool all_near(int lanes, int F) { return lanes * (F + 128) > 20 * F; }
+
+// The term of triangle j for this lane's point, rounded as near_pairs rounds it:
+// the pairs in eight sums, added in the order of its shuffles.  The nodes come
+// through `stage`, kPairStage pairs at a time, a lane loading one float4 of them: as
+// broadcasts from global memory they keep the L1 busy (31.4 ms for 100,000 points
+// near to all of 1,280 triangles at level 3, 22.1 ms like this).
+__device__ __forceinline__ float near_term(const CvGeom& c, int j, float3 x, const NegPoint2& nx,
+                                           float4* stage)
+{
+    const int lane = threadIdx.x & 31, pairs = c.F >> 1;
+    const float4 tp = __ldg(c.tri_p + j);
+    const float4* nd = c.fine_pk + (int64_t)c.F * j;
+    float2 unused = make_float2(0.f, 0.f);
+    if (c.F == kCoarse) {  // level 0: three pairs and the odd node
+        float2 s[3];
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+            s[u] = make_float2(0.f, 0.f);
+            node_acc2<false>(__ldg(nd + 2 * u), __ldg(nd + 2 * u + 1), unused, nx, s[u], unused);
+        }
+        float odd = 0.f, zero = 0.f;
+        node_acc(__ldg(nd + 6), 0.f, x, odd, zero);
+        const float v = ((s[0].x + s[0].y) + (s[2].x + s[2].y)) + ((s[1].x + s[1].y) + odd);
+        return tri_term(tp, 0.f, x, 0.f, v, 0.f, 0.f);
+    }
+    float2 s[kPairLanes];
+#pragma unroll
+    for (int u = 0; u < kPairLanes; ++u) s[u] = make_float2(0.f, 0.f);
+    float4 next = __ldg(nd + min(lane, 2 * pairs - 1));
+    for (int q0 = 0; q0 < pairs; q0 += kPairStage) {
+        __syncwarp();  // the previous pairs are no longer read
+        stage[lane] = next;
+        next = __ldg(nd + min(2 * (q0 + kPairStage) + lane, 2 * pairs - 1));
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < kPairStage; h += kPairLanes)
+            if (q0 + h < pairs) {
+#pragma unroll
+                for (int u = 0; u < kPairLanes; ++u)
+                    if (q0 + h + u < pairs)
+                        node_acc2<false>(stage[2 * (h + u)], stage[2 * (h + u) + 1], unused, nx, s[u],
+                                         unused);
+            }
+    }
+    float v[kPairLanes];
+#pragma unroll
+    for (int u = 0; u < kPairLanes; ++u) v[u] = s[u].x + s[u].y;
+#pragma unroll
+    for (int o = kPairLanes / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int u = 0; u < o; ++u) v[u] += v[u + o];
+    return tri_term(tp, 0.f, x, 0.f, v[0], 0.f, 0.f);
+}
+
+template <int SPLIT>
 __global__ void __launch_bounds__(32 * kPointWarps, 4) k_cv_quad_D(CvGeom c, const float* __restrict__ x,
-                                                                int64_t n, float* out)
+                                                                   int64_t n, float* out)
 {
     __shared__ PointTile sm;
+    constexpr int kPoints = 32 * kPointWarps / SPLIT;  // of a block
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int kShare = kPointTris / 2 / kPointWarps;  // records of a tile per warp
     const float om[kCoarse] = {};
     int* queue = sm.queue[warp];
-    for (int64_t base = 32 * (int64_t)blockIdx.x; base < n; base += 32 * (int64_t)gridDim.x) {
-        const int64_t i = base + lane;
+    for (int64_t base = kPoints * (int64_t)blockIdx.x; base < n; base += kPoints * (int64_t)gridDim.x) {
+        const int64_t i = base + 32 * (warp / SPLIT) + lane;
         const bool ok = i < n;
         const float3 p = ok ? make_float3(x[3 * i], x[3 * i + 1], x[3 * i + 2])
                             : make_float3(0.f, 0.f, 0.f);
@@ -525,15 +597,26 @@ __global__ void __launch_bounds__(32 * kPointWarps, 4) k_cv_quad_D(CvGeom c, con
         double tot = 0.0;
         ff near_tot = {0.f, 0.f};
         int queued = 0;
+        auto visit = [&](bool near, int j) {
+            const unsigned b = __ballot_sync(0xFFFFFFFFu, near);
+            if (all_near(__popc(b), c.F)) {
+                const float v = near_term(c, j, p, nx, sm.fine[warp]);
+                if (near) add_near(near_tot, v);
+            } else {
+                if (near) queue[queued + __popc(b & ((1u << lane) - 1))] = lane << 20 | j;
+                queued += __popc(b);
+            }
+        };
         for (int j0 = 0; j0 < c.T; j0 += kPointTris) {
             const int recs = (min(kPointTris, c.T - j0) + 1) >> 1;
             __syncthreads();  // the previous tile is no longer read
             for (int k = threadIdx.x; k < recs * kFarRec; k += blockDim.x)
                 sm.rec[k] = __ldg(c.far + (int64_t)(j0 >> 1) * kFarRec + k);
             __syncthreads();
+            const int share = (recs + SPLIT - 1) / SPLIT;
+            const int begin = (warp % SPLIT) * share, end = min(recs, begin + share);
             float part = 0.f;
-            const int end = min(recs, (warp + 1) * kShare);
-            for (int r = warp * kShare; r < end; ++r) {
+            for (int r = begin; r < end; ++r) {
                 const int j = j0 + 2 * r;
                 bool near0, near1;
                 const float2 term = far_pair<false>(sm.rec + r * kFarRec, om, nx, 0.f, near0, near1);
@@ -542,28 +625,31 @@ __global__ void __launch_bounds__(32 * kPointWarps, 4) k_cv_quad_D(CvGeom c, con
                 near0 = near0 && ok;
                 near1 = near1 && ok && j + 1 < c.T;
                 if (__any_sync(0xFFFFFFFFu, near0 || near1)) {
-                    const unsigned b0 = __ballot_sync(0xFFFFFFFFu, near0),
-                                   b1 = __ballot_sync(0xFFFFFFFFu, near1), below = (1u << lane) - 1;
-                    if (near0) queue[queued + __popc(b0 & below)] = lane << 20 | j;
-                    queued += __popc(b0);
-                    if (near1) queue[queued + __popc(b1 & below)] = lane << 20 | (j + 1);
-                    queued += __popc(b1);
+                    visit(near0, j);
+                    visit(near1, j + 1);
                     if (queued > kPairQueue - 64) {
                         near_pairs(c, queue, queued, p, near_tot);
                         queued = 0;
                     }
                 }
+                if (SPLIT < kPointWarps && r % kPointRun == kPointRun - 1) {
+                    tot += (double)part;
+                    part = 0.f;
+                }
             }
             tot += (double)part;
         }
         near_pairs(c, queue, queued, p, near_tot);
-        sm.sum[warp][lane] = tot + ((double)near_tot.hi + (double)near_tot.lo);
-        __syncthreads();
-        if (warp == 0 && ok) {
-            for (int k = 1; k < kPointWarps; ++k) tot = k == 1 ? sm.sum[0][lane] + sm.sum[1][lane] : tot + sm.sum[k][lane];
-            out[i] = (float)(tot * (double)kInvFourPi);
+        tot += (double)near_tot.hi + (double)near_tot.lo;
+        if (SPLIT > 1) {
+            __syncthreads();  // (the sums take the place of the stages)
+            sm.sum[warp][lane] = tot;
+            __syncthreads();
+            if (warp % SPLIT == 0)
+                for (int k = 1; k < SPLIT; ++k) tot += sm.sum[warp + k][lane];
         }
-        __syncthreads();
+        if (ok && warp % SPLIT == 0) out[i] = (float)(tot * (double)kInvFourPi);
+        if (SPLIT > 1) __syncthreads();
     }
 }
 
@@ -939,11 +1025,21 @@ void free_cv(wob_cv_s* c)
         if (p) cudaFree(p);
 }
 
+// Warps of a set of 32 points.  Eight share the triangles until there are points
+// for about two rounds of blocks with a set per warp; 300,000 points on 20, 80 and
+// 1,280 triangles take 0.76, 0.96 and 0.99 of the time so, 100,000 0.95, 1.07 and
+// 1.13.  A boundary of one or two records a warp (level 0) is worth it at a third of
+// that: 100,000 points on 20 triangles 20.7 us against 26.9.
 cudaError_t launch_quad_D(const CvGeom& g, const float* x, int64_t n, float* out, cudaStream_t s)
 {
     const int threads = 32 * kPointWarps;
-    k_cv_quad_D<<<grid_for((const void*)k_cv_quad_D, threads, 0, n * kPointWarps), threads, 0, s>>>(
-        g, x, n, out);
+    const int64_t blocks = (n + threads - 1) / threads;  // with a set per warp
+    const int64_t full = grid_for((const void*)k_cv_quad_D<1>, threads, 0, INT64_MAX / 2);
+    if (10 * blocks >= (g.T * (int64_t)g.F <= 256 ? 6 : 19) * full)
+        k_cv_quad_D<1><<<(int)(blocks < full ? blocks : full), threads, 0, s>>>(g, x, n, out);
+    else
+        k_cv_quad_D<kPointWarps><<<grid_for((const void*)k_cv_quad_D<kPointWarps>, threads, 0, n * kPointWarps),
+                                   threads, 0, s>>>(g, x, n, out);
     return cudaGetLastError();
 }
 
