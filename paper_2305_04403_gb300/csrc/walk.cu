@@ -600,6 +600,11 @@ __global__ void __launch_bounds__(128, WOB_SL_MIN_BLOCKS) k_sl_walks_ff(WalkPara
 // lanes that stayed or had another condition branched apart (16 of 32 active).
 // ---------------------------------------------------------------------------
 
+// A query further than this many L from the boundary takes its own distance as
+// the unit of length for its step: in units of L its r^2 leaves FP32's range, and
+// 1 / r loses its low part before.
+constexpr float kRisFar = 0x1p30f;
+
 // 1 / sqrt(a) for a normal a: the fast root y, corrected to second order in
 // e = 1 - a y^2 (y (1 + e / 2 + 3 e^2 / 8); e ~ 1e-7).
 __device__ __forceinline__ ff ff_rsqrt(ff a)
@@ -608,6 +613,12 @@ __device__ __forceinline__ ff ff_rsqrt(ff a)
     const ff t = ff_mul(a, two_prod(y, y));
     const float e = rn_sub(rn_sub(1.f, t.hi), t.lo);
     return fast_two_sum(y, rn_mul(rn_mul(y, e), rn_fma(0.375f, e, 0.5f)));
+}
+
+// 2^-e for 2^e <= d < 2^(e + 1), within FP32's normal range.
+__device__ __forceinline__ float unit_of(float d)
+{
+    return __int_as_float(max(254 - (__float_as_int(d) >> 23), 1) << 23);
 }
 
 // K without its constant factor, at the candidate y of the vertex x (condition
@@ -698,7 +709,7 @@ __global__ void __launch_bounds__(kRisThreads, kRisBlocks) k_sl_walks_ris(WalkPa
     const int64_t total = p.Q * (int64_t)p.N;
     const double phi = (double)p.phi;
     const int se = ilogb(p.L);
-    const float scale = scalbnf(1.f, -se), alpha = p.alpha / scale;
+    const float unit = scalbnf(1.f, -se), alpha = p.alpha / unit;
     // |Gamma| / ris times the constant factors of K and the units' powers, and each
     // walk's sums and normal: in shared memory, off the candidates' registers (71 of
     // them hold the loop without spills)
@@ -707,10 +718,10 @@ __global__ void __launch_bounds__(kRisThreads, kRisBlocks) k_sl_walks_ris(WalkPa
     __shared__ double weight[3], walk[3][kRisThreads];
     __shared__ volatile float normal[6][kRisThreads];  // n_x
     if (threadIdx.x == 0) {
-        const double wq = p.area / (double)p.ris / kFourPi * (double)scale;  // G
+        const double wq = p.area / (double)p.ris / kFourPi * (double)unit;   // G
         weight[kQueryW] = wq;
         weight[kDirichletW] = wq * ((double)p.kmix / (double)p.pk);          // (k / p_k) G
-        weight[kLayerW] = 2.0 * wq * (double)scale;                          // 2 dG/dn_x
+        weight[kLayerW] = 2.0 * wq * (double)unit;                           // 2 dG/dn_x
     }
     __syncthreads();
     const int uniform_bc = p.kind == WOB_ROBIN_SL ? WOB_BC_ROBIN : WOB_BC_NEUMANN;
@@ -725,14 +736,18 @@ __global__ void __launch_bounds__(kRisThreads, kRisBlocks) k_sl_walks_ris(WalkPa
         const int64_t wi = live ? idx - qi * p.N : 0;
         const uint32_t q = p.q_base + (uint32_t)qi;
         const uint32_t w = (uint32_t)(p.walk_begin + wi);
+        const float* vertex = p.verts + 3 * (int64_t)__ldg(p.tris);
+        float dist = 0.f;  // of the query from the boundary
         FFPoint x;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             x.v0[c] = p.queries[3 * qi + c];
+            dist = fmaxf(dist, fabsf(x.v0[c] - __ldg(vertex + c)));
             x.p[c] = {0.f, 0.f};
             x.n[c] = {0.f, 0.f};
             normal[2 * c][threadIdx.x] = normal[2 * c + 1][threadIdx.x] = 0.f;
         }
+        float scale = dist * unit > kRisFar ? unit_of(dist) : unit;
         int bx = -1;
         int32_t jx = -1;
         float ux = 0.f, u2x = 0.f;
@@ -798,7 +813,11 @@ __global__ void __launch_bounds__(kRisThreads, kRisBlocks) k_sl_walks_ris(WalkPa
                     // parts, negative on Dirichlet parts (and for a zero kernel)
                     const float sg = bx < 0 ? wc[pick].hi : bx == WOB_BC_DIRICHLET ? -1.f
                                                           : -(float)p.phi * wc[pick].hi;
-                    const double wk = weight[bx < 0 ? kQueryW : bx == WOB_BC_DIRICHLET ? kDirichletW : kLayerW];
+                    double wk = weight[bx < 0 ? kQueryW : bx == WOB_BC_DIRICHLET ? kDirichletW : kLayerW];
+                    if (scale != unit) {  // a far query's step is over
+                        wk *= (double)scale / (double)unit;
+                        scale = unit;
+                    }
                     wfac = (sg > 0.f ? wk : -wk) * ff_join(sumw);
                     x = y;
 #pragma unroll
