@@ -702,28 +702,36 @@ __device__ __forceinline__ double ris_data(const WalkParams& p, int64_t j, const
     return bc == WOB_BC_ROBIN ? dhdn + (double)p.alpha * (double)h : dhdn;
 }
 
+// The unit of length and |Gamma| / ris times the constant factors of K and the
+// unit's powers.  Formed by the host: as three FP64 quotients in a row in the first
+// thread of each block they took 2 of the 8.9 us of a call of two walks.
+struct RisUnits {
+    float unit, alpha;               // 1 / length; alpha in it
+    double query, dirichlet, layer;  // G, (k / p_k) G, 2 dG/dn_x
+};
+
+RisUnits ris_units(const WalkParams& p)
+{
+    RisUnits u;
+    u.unit = std::ldexp(1.f, -std::ilogb(p.L));
+    u.alpha = p.alpha / u.unit;
+    u.query = p.area / (double)p.ris / kFourPi * (double)u.unit;
+    u.dirichlet = u.query * ((double)p.kmix / (double)p.pk);
+    u.layer = 2.0 * u.query * (double)u.unit;
+    return u;
+}
+
 template <bool DEBUG>
-__global__ void __launch_bounds__(kRisThreads, kRisBlocks) k_sl_walks_ris(WalkParams p)
+__global__ void __launch_bounds__(kRisThreads, kRisBlocks) k_sl_walks_ris(WalkParams p, RisUnits ru)
 {
     const StreamKey key{p.key0, p.key1};
     const int64_t total = p.Q * (int64_t)p.N;
     const double phi = (double)p.phi;
-    const int se = ilogb(p.L);
-    const float unit = scalbnf(1.f, -se), alpha = p.alpha / unit;
-    // |Gamma| / ris times the constant factors of K and the units' powers, and each
-    // walk's sums and normal: in shared memory, off the candidates' registers (71 of
-    // them hold the loop without spills)
-    enum { kQueryW, kDirichletW, kLayerW };
+    const float unit = ru.unit, alpha = ru.alpha;
+    // each walk's sums and normal: in shared memory, off the candidates' registers
     enum { kSum, kProduct, kFirst };
-    __shared__ double weight[3], walk[3][kRisThreads];
+    __shared__ double walk[3][kRisThreads];
     __shared__ volatile float normal[6][kRisThreads];  // n_x
-    if (threadIdx.x == 0) {
-        const double wq = p.area / (double)p.ris / kFourPi * (double)unit;   // G
-        weight[kQueryW] = wq;
-        weight[kDirichletW] = wq * ((double)p.kmix / (double)p.pk);          // (k / p_k) G
-        weight[kLayerW] = 2.0 * wq * (double)unit;                           // 2 dG/dn_x
-    }
-    __syncthreads();
     const int uniform_bc = p.kind == WOB_ROBIN_SL ? WOB_BC_ROBIN : WOB_BC_NEUMANN;
     ff wc[kMaxRis];
     const int lane = threadIdx.x & 31;
@@ -813,7 +821,7 @@ __global__ void __launch_bounds__(kRisThreads, kRisBlocks) k_sl_walks_ris(WalkPa
                     // parts, negative on Dirichlet parts (and for a zero kernel)
                     const float sg = bx < 0 ? wc[pick].hi : bx == WOB_BC_DIRICHLET ? -1.f
                                                           : -(float)p.phi * wc[pick].hi;
-                    double wk = weight[bx < 0 ? kQueryW : bx == WOB_BC_DIRICHLET ? kDirichletW : kLayerW];
+                    double wk = bx < 0 ? ru.query : bx == WOB_BC_DIRICHLET ? ru.dirichlet : ru.layer;
                     if (scale != unit) {  // a far query's step is over
                         wk *= (double)scale / (double)unit;
                         scale = unit;
@@ -1533,9 +1541,9 @@ int launch_sl_walks(const WalkParams& p, bool debug, cudaStream_t s)
     const int64_t work = p.Q * (int64_t)p.N;
     if (p.ris > 1) {
         if (debug)
-            k_sl_walks_ris<true><<<grid_for((const void*)k_sl_walks_ris<true>, threads, 0, work), threads, 0, s>>>(p);
+            k_sl_walks_ris<true><<<grid_for((const void*)k_sl_walks_ris<true>, threads, 0, work), threads, 0, s>>>(p, ris_units(p));
         else
-            k_sl_walks_ris<false><<<grid_for((const void*)k_sl_walks_ris<false>, threads, 0, work), threads, 0, s>>>(p);
+            k_sl_walks_ris<false><<<grid_for((const void*)k_sl_walks_ris<false>, threads, 0, work), threads, 0, s>>>(p, ris_units(p));
     } else if (debug) {
         k_sl_walks_ff<true><<<grid_for((const void*)k_sl_walks_ff<true>, threads, 0, work), threads, 0, s>>>(p);
     } else {
