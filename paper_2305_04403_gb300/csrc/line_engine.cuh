@@ -196,6 +196,15 @@ __device__ __forceinline__ int pick_hit(const float4* __restrict__ tv, const int
     return bpos;
 }
 
+// The node phase goes on while this many eighths of the live lanes have nodes to
+// visit: one (until the last lane is done) in trees of up to six levels, where a
+// line's visits differ by little and the landing phase counts for more, two in
+// deeper ones.  At four, with which lanes land sooner but fewer together, 1.05e6
+// walks of four lines took 1.26, 1.09, 0.98, 0.93, 0.85 and 0.76 of the lock-step
+// time on 2 to 7 levels (20 to 81,920 triangles), and take 1.04, 0.88, 0.83, 0.86,
+// 0.79 and 0.70 with this rule.
+__device__ __forceinline__ int line_busy_eighths(int levels) { return levels <= 6 ? 1 : 2; }
+
 // Run the policy's walks to the end.  The policy P provides
 //   bool fetch(int slot, int& cnt)     (whole warp) the next tile into slot
 //   StreamKey key(const LaneWalk&)     streams of the lane's problem
@@ -210,6 +219,7 @@ template <class P, bool COUNT>
 __device__ __forceinline__ void run_lines(P& pol, const LaneMem mem, double* block_vals, int levels,
                                           int& err, WalkCount& c)
 {
+    const int busy_eighths = line_busy_eighths(levels);
     const int lane = threadIdx.x & 31;
     double* vals = block_vals + 2 * (threadIdx.x & ~31);  // of the warp's two tiles
     unsigned todo0 = 0, todo1 = 0;  // unfinished walks of the tile slots
@@ -277,7 +287,7 @@ __device__ __forceinline__ void run_lines(P& pol, const LaneMem mem, double* blo
         const float oix = mem.x_hi(0) * ix, oiy = mem.x_hi(1) * iy, oiz = mem.x_hi(2) * iz;
         // ---- nodes
         const int n_live = __popc(livem);
-        const int need = (n_live + 1) >> 1;
+        const int need = (n_live * busy_eighths + 7) >> 3;
         while (true) {
             const bool can = trav && nq < kNodeQ;
             const unsigned busy = __ballot_sync(kAllLanes, can);
