@@ -394,9 +394,6 @@ __device__ __forceinline__ void binary_children(const float4* __restrict__ nodes
     b.lo[0] = n1.x; b.hi[0] = n1.y; b.lo[1] = n1.z; b.hi[1] = n1.w; b.lo[2] = n2.z; b.hi[2] = n2.w;
 }
 
-// One level of the collapse.  counts[i]: wide nodes of level i, counted from the
-// level whose first node is `first`; this launch does level `level` of these
-// and counts the next one, whose nodes follow its own.
 // (a - org) s for a >= org and a power of two s, rounded down (up) to a whole
 // number, exactly: the difference as a sum of two floats (two-sum), whose low
 // part moves the floor (ceiling) only where the high part is whole.
@@ -413,6 +410,9 @@ __device__ __forceinline__ int quantise_up(float a, float org, float s)
     return (int)f + (f == v && (d.lo > 0.f || (v == 0.f && d.hi > 0.f)));
 }
 
+// One level of the collapse.  counts[i]: wide nodes of level i, counted from the
+// level whose first node is `first`; this launch does level `level` of these
+// and counts the next one, whose nodes follow its own.
 __global__ void k_wide_collapse(const float4* __restrict__ nodes, int root_ref, float3 root_lo,
                                 float3 root_hi, int64_t first, int level, int* __restrict__ counts,
                                 int32_t* __restrict__ src, float4* __restrict__ wn)

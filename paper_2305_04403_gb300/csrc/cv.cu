@@ -352,7 +352,7 @@ __device__ __forceinline__ float fine_tri(const CvGeom& c, int j, float3 x, floa
 // rounded as the scalar operations round it, nodes 0, 2, 4 and 1, 3, 5 in two
 // sums that meet before node 6.  VALUE: fx counts (else 0, and S0 is not formed).
 // Bounded by the FMA pipe: 80 packed operations (two cycles each) for 63
-// instructions a triangle: 3.6 of the 7.15 ms (9.5 before) that the residual walks
+// instructions a triangle: 3.6 of the 7.12 ms (9.5 before) that the residual walks
 // of 8,192 queries x 64 walks x 2 vertices take, the fine nodes 2.3.  A form with the
 // centroid's distance and offsets along two medians needs 30% fewer operations,
 // and rounds differently.
@@ -762,10 +762,8 @@ __global__ void __launch_bounds__(128, 4) k_cvw_trace(WalkParams p, CvWalk st, i
         const float Tthr = p.edge_thr_L * fabsf(L.Sz);
         Trav t;
         trav_init(t);
-        uint32_t nn = 0, nt = 0;
-        trace_wide<false, false>(p.nodes, p.tv, L, make_float3(0.f, 0.f, 0.f), Tthr, p.tauL,
-                                 p.graze, self, t, hits, stack, key, q, w, (uint32_t)k, nn, nt,
-                                 err, p.iter_limit);
+        trace_wide<false>(p.nodes, p.tv, L, make_float3(0.f, 0.f, 0.f), Tthr, p.tauL, p.graze, self, t,
+                          hits, stack, key, q, w, (uint32_t)k, err, p.iter_limit);
         if (t.m == 0) {
             st.alive[i] = 0;
             st.own[i] = kSubs * st.T;
@@ -898,10 +896,8 @@ __global__ void __launch_bounds__(128, 4) k_cvmc_lines(WalkParams p, CvWalk st, 
         const float Tthr = p.edge_thr_L * fabsf(L.Sz);
         Trav tr;
         trav_init(tr);
-        uint32_t nn = 0, nt = 0;
-        trace_wide<false, false>(p.nodes, p.tv, L, make_float3(0.f, 0.f, 0.f), Tthr, p.tauL,
-                                 p.graze, st.self[i], tr, hits, stack, key, q, w, step, nn, nt,
-                                 err, p.iter_limit);
+        trace_wide<false>(p.nodes, p.tv, L, make_float3(0.f, 0.f, 0.f), Tthr, p.tauL, p.graze,
+                          st.self[i], tr, hits, stack, key, q, w, step, err, p.iter_limit);
         if (tr.m == 0) {
             mc.wgt[t] = 0.f;
             pp[0] = pp[1] = pp[2] = 0.f;

@@ -9,16 +9,16 @@
 //   hand out   lanes without a walk take the next one of the warp's tiles;
 //   axis       lanes that begin a line draw its axis;
 //   nodes      lanes with nodes left visit them, one node per lane and turn,
-//              until fewer than `need` lanes have work;
+//              until fewer than `need` lanes have work (line_busy_eighths);
 //   leaves     the queued leaf triangles are tested;
 //   land       lanes whose traversal is complete pick their hit, refine it
 //              and add its term (the walk's own arithmetic, in the policy),
 // and a lane that lands begins its next line while the others go on with
-// theirs.  Waiting until half of the lanes have finished makes the
-// landing phase (about 700 instructions) serve a dozen lanes at a time and
-// keeps most lanes busy in the node phase, which has nine tenths of the work.  Everything a lane does for its own walk is the same
-// arithmetic in the same order whatever the other lanes do, so the values
-// of the walks do not depend on the schedule.
+// theirs.  Waiting until most lanes have finished lets the landing phase
+// (about 700 instructions) serve some two dozen lanes at a time, while the
+// longest traversals go on beside the next lines.  Everything a lane does for
+// its own walk is the same arithmetic in the same order whatever the other
+// lanes do, so the values of the walks do not depend on the schedule.
 //
 // Tiles: a warp owns up to two tiles of 32 consecutive walks at a time (the
 // one being handed out and the one whose last walks are still under way);
@@ -31,16 +31,14 @@
 // line, the node, the queue and stack heights in registers.
 //
 // Measured against one thread per walk in lock step: the level-6 star slice
-// (60.4 M lines: 7,374 queries x 512 walks x 16) 64.7 -> 41.9 ms, direct-BIE
-// walks on the 200,000-triangle torus 40.1 -> 21.4 ms, 24 batched problems
-// 31.3 -> 19.6 ms; 978 -> 579 warp instructions a line and 10.8 -> 15.8 lanes
+// (60.4 M lines: 7,374 queries x 512 walks x 16) 64.7 -> 39.5 ms, direct-BIE
+// walks on the 200,000-triangle torus 40.1 -> 20.0 ms, 24 batched problems
+// 31.3 -> 17.8 ms; 978 -> 532 warp instructions a line and 10.8 -> 17.3 lanes
 // an instruction on the slice.  What bounds it now is the instruction issue
-// (59% of cycles; L1 53%).  With `need` at 7, 5, 4, 3, 1 eighths of the live
-// lanes an earlier form took 60.6, 48.4, 45.9, 46.7 and 48.0 ms; with leaf
-// references queued instead of (node, slots) entries 45.9 against 44.7 ms;
-// with 16-byte instead of 32-byte node loads 44.7 against 44.0 ms; with 5 and
-// 7 instead of 6 blocks per SM 46.6 and (values in local memory) 49.4 against
-// 41.9 ms.
+// (63% of cycles; L1 58%).  Earlier forms, on the slice: leaf references queued
+// instead of (node, slots) entries 45.9 against 44.7 ms; 16-byte instead of
+// 32-byte node loads 44.7 against 44.0 ms; 5 and 7 instead of 6 blocks per SM
+// 46.6 and (values in local memory) 49.4 against 41.9 ms.
 #pragma once
 
 #include "node_stack.cuh"
@@ -406,9 +404,11 @@ __device__ __forceinline__ void run_lines(P& pol, const LaneMem mem, double* blo
 // instructions and a call of a few thousand walks has G times the warps; the
 // price is the landing phase, which runs on one lane of G.  Same box and
 // triangle tests, same hits, same arithmetic per walk: the same values.
-// 16,384 walks of 4 lines on 1,280 triangles take 151 us with a lane per walk
-// and 100, 92 and 113 us with 2, 4 and 8 lanes (two warps of four lanes each
-// for every walk's warp, without splitting the nodes: 169 us).
+// 16,384 walks of 4 lines on 1,280 triangles take 90 us; with the stack shared
+// by the group and a barrier between its pop and its push 97 us, and in that form
+// without the barrier 92 us against 151 with a lane per walk, 100 with 2 lanes and
+// 113 with 8 (two warps of four lanes each for every walk's warp, without
+// splitting the nodes: 169 us).
 // ---------------------------------------------------------------------------
 constexpr int kG = 4;                       // lanes per walk: 2, 4 or 8
 constexpr int kGroups = 32;                 // walks of a block: one tile

@@ -35,15 +35,15 @@ constexpr double kFourPi = 12.566370614359172953850573533118;
 // line_engine.cuh), 24 warps of the grouped form; the forms that need more
 // registers than that to keep out of local memory get fewer blocks.
 constexpr int kLineBlocks = 6;
-constexpr int kNdBlocks = 7;  // direct BIE: 72 registers hold it (22.7 -> 21.4 ms on the torus)
+constexpr int kNdBlocks = 7;  // direct BIE: 72 registers hold it (20.0 ms on the torus; the step from 6 was 6%)
 constexpr int kDebugBlocks = 4;
 constexpr int kGroupBlocks = 24 / kG;
 // Calls of at most this many walks per SM run with a group of lanes per walk.
-// 32,768 walks (216 per SM) took the group and the single lane 150 and 158 us
-// (4 lines each, 1,280 triangles), 1,318 and 1,262 us (16 lines, 81,920) and
-// 1,035 and 997 us (direct BIE, 12 lines); half as many 98 against 153, 772
-// against 1,160 and 633 against 938 us; twice as many 226 against 205, 2,064
-// against 1,454 and 1,608 against 1,153 us.
+// 32,768 walks (216 per SM) take the group and the single lane 141 and 139 us
+// (4 lines each, 1,280 triangles), 1,316 and 1,149 us (16 lines, 81,920) and
+// 1,033 and 911 us (direct BIE, 12 lines); half as many 88 against 131, 753
+// against 1,040 and 587 against 897 us; twice as many 213 against 168, 2,083
+// against 1,347 and 1,610 against 1,077 us.
 constexpr int64_t kGroupWalksPerSm = 200;
 // Single-layer walks with area sampling: 7 blocks of 128 threads per SM (72
 // registers, no spills) hide the latency of the CDF search: 4.31 ms for 2.0e8

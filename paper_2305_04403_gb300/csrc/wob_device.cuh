@@ -511,30 +511,20 @@ __device__ __forceinline__ int pick4(int4 v, int j)
 // postponed leaves, speculative traversal).  A leaf that does not fit in
 // the queue is tested on the spot.  The set of triangles tested is the
 // same as with immediate tests.
-// 15 entries: with the 8 KB of parked walk state a 128-thread block holds
-// 15.5 KB of shared memory, so eight blocks (each with 1 KB reserved) fit
-// the 132 KB shared-memory carveout and leave 124 KB of L1 per SM (16
-// entries need the 164 KB carveout, 92 KB of L1, and run 3% slower).
+// 15 entries, in local memory (the walks of line_engine.cuh have their own
+// driver): in a walk kernel of this form 8 entries took 3% and 32 entries 1% more
+// than 16.
 constexpr int kLeafQ = 15;
 
-// Where a lane keeps its queued leaf triangles: entry i at base[i * stride]
-// (shared memory, structure of arrays, in the walk kernels; a local array
-// elsewhere).
-struct LeafQueue {
-    int* base;
-    int stride;
-    __device__ __forceinline__ int& operator[](int i) const { return base[i * stride]; }
-};
-
-template <bool COUNT, bool SUM_S>
-__device__ __forceinline__ void trace_wide_q(const float4* __restrict__ wn,
-                                             const float4* __restrict__ tv, const LinePre& L,
-                                             float3 d, float Tthr, float tauL, float graze,
-                                             int exclude_pos, Trav& t, int* hits, int* stack,
-                                             StreamKey key, uint32_t q, uint32_t walk,
-                                             uint32_t step, uint32_t& n_nodes, uint32_t& n_tris,
-                                             int& err, int iter_limit, LeafQueue lq)
+template <bool SUM_S>
+__device__ __forceinline__ void trace_wide(const float4* __restrict__ wn,
+                                           const float4* __restrict__ tv, const LinePre& L,
+                                           float3 d, float Tthr, float tauL, float graze,
+                                           int exclude_pos, Trav& t, int* hits, int* stack,
+                                           StreamKey key, uint32_t q, uint32_t walk,
+                                           uint32_t step, int& err, int iter_limit)
 {
+    int lq[kLeafQ];
     int node = 0, sp = 0, iters = 0, nq = 0;
     bool done = false;
     while (true) {
@@ -558,7 +548,6 @@ __device__ __forceinline__ void trace_wide_q(const float4* __restrict__ wn,
                 done = true;
                 break;
             }
-            if (COUNT) n_nodes++;
             const float4* nd = wn + 6 * node;
             const float4 h = __ldg(nd);
             const int nint = (__float_as_uint(h.w) >> 24) & 15;
@@ -580,7 +569,6 @@ __device__ __forceinline__ void trace_wide_q(const float4* __restrict__ wn,
                         if (nq < kLeafQ) {
                             lq[nq++] = p;
                         } else {
-                            if (COUNT) n_tris++;
                             test_tri<SUM_S>(tv, L, d, Tthr, tauL, graze, p, t, hits, key, q,
                                             walk, step);
                         }
@@ -603,26 +591,11 @@ __device__ __forceinline__ void trace_wide_q(const float4* __restrict__ wn,
         }
         // the queued triangles, all lanes together
         for (int i = 0; i < nq; ++i) {
-            if (COUNT) n_tris++;
             test_tri<SUM_S>(tv, L, d, Tthr, tauL, graze, lq[i], t, hits, key, q, walk, step);
         }
         nq = 0;
         if (done) break;
     }
-}
-
-template <bool COUNT, bool SUM_S>
-__device__ __forceinline__ void trace_wide(const float4* __restrict__ wn,
-                                           const float4* __restrict__ tv, const LinePre& L,
-                                           float3 d, float Tthr, float tauL, float graze,
-                                           int exclude_pos, Trav& t, int* hits, int* stack,
-                                           StreamKey key, uint32_t q, uint32_t walk,
-                                           uint32_t step, uint32_t& n_nodes, uint32_t& n_tris,
-                                           int& err, int iter_limit)
-{
-    int lq[kLeafQ];
-    trace_wide_q<COUNT, SUM_S>(wn, tv, L, d, Tthr, tauL, graze, exclude_pos, t, hits, stack, key,
-                               q, walk, step, n_nodes, n_tris, err, iter_limit, LeafQueue{lq, 1});
 }
 
 // The picked hit (leaf position) after the traversal; -1 if m == 0.
@@ -656,10 +629,9 @@ __device__ __forceinline__ int trace_line(const float4* __restrict__ nodes,
     const float Tthr = edge_thr_L * fabsf(L.Sz);
     int stack[kStackSize];
     int hits[kMaxHits];
-    uint32_t nn = 0, nt = 0;
     trav_init(t);
-    trace_wide<false, SUM_S>(nodes, tv, L, d, Tthr, tauL, graze, exclude_pos, t, hits, stack, key,
-                             q, walk, step, nn, nt, err, iter_limit);
+    trace_wide<SUM_S>(nodes, tv, L, d, Tthr, tauL, graze, exclude_pos, t, hits, stack, key, q, walk,
+                      step, err, iter_limit);
     return select_hit(tv, t, hits, key, q, walk, step);
 }
 
