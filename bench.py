@@ -43,15 +43,15 @@ X0 = (3.0, 0.0, 0.0)
 # data term and accumulation), and the bytes fetched per node and triangle.
 OPS_NODE, OPS_TRI, OPS_HIT, OPS_LINE = 320, 41, 100, 585
 BYTES_NODE, BYTES_TRI = 96, 48
-# DRAM bytes (read + write) of one full-size k_dl_walks launch of this
+# DRAM bytes (read + write) of one full-size k_dl_lines launch of this
 # workload (queries, leaf size, bytes) from ncu dram__bytes_read.sum +
-# dram__bytes_write.sum (profiles/k_dl_walks_star6_wide.md); None while the
+# dram__bytes_write.sum (profiles/k_dl_lines_star6.md); None while the
 # kernel has changed since the last capture.
-TRAFFIC_FULL = (29497, 1, 27.07e6 + 135.12e6)
+TRAFFIC_FULL = (29497, 1, 22.18e6 + 0.37e6)
 # The walk kernel's issue-slot use from the same profile: fraction of cycles
 # with an instruction issued, and active threads per warp instruction; None
 # while the kernel has changed since the last capture.
-ISSUE_PROFILE = (0.722, 10.77)
+ISSUE_PROFILE = (0.635, 17.28)
 
 
 def _peaks():
@@ -288,7 +288,7 @@ def run_ours(args):
                      "unit": "GB/s", "frac": achieved_gbs / hbm,
                      "traffic": (TRAFFIC_FULL[2] if TRAFFIC_FULL and
                                  (Q, args.leaf) == TRAFFIC_FULL[:2] else None),
-                     "kernel": "k_dl_walks",
+                     "kernel": "k_dl_lines",
                      "algorithmic_bytes_per_launch": bytes_step,
                      "bytes_per_unit": {"wide_node": BYTES_NODE, "triangle": BYTES_TRI},
                      "peak_source": f"MEASURED_PEAKS.json hbm_gbs ({which})",
