@@ -17,6 +17,7 @@
 // tensor cores), then quadrature + accumulation (one thread per walk; the
 // far-field loop over triangles is the same for every lane of a warp, so its
 // node loads are broadcasts).
+#include <algorithm>
 #include <array>
 #include <climits>
 #include <cmath>
@@ -471,6 +472,7 @@ __device__ __forceinline__ float quad_sum(const CvGeom& c, FarTile& sm, float3 x
 // points the queue took 368 us, the form before it 23 and this one 21 (level 0).
 constexpr int kPointWarps = 8, kPointTris = 256, kPairQueue = 128, kPairLanes = 8;
 constexpr int kPointRun = kPointTris / 2 / kPointWarps;
+constexpr int kPointBlocks = 4;  // per SM: 64 registers, 47 KB of shared memory
 constexpr int kPairStage = 16;  // pairs of nodes that a warp stages for all its lanes
 struct PointTile {
     float4 rec[kPointTris / 2 * kFarRec];
@@ -580,7 +582,7 @@ __device__ __forceinline__ float near_term(const CvGeom& c, int j, float3 x, con
 }
 
 template <int SPLIT>
-__global__ void __launch_bounds__(32 * kPointWarps, 4) k_cv_quad_D(CvGeom c, const float* __restrict__ x,
+__global__ void __launch_bounds__(32 * kPointWarps, kPointBlocks) k_cv_quad_D(CvGeom c, const float* __restrict__ x,
                                                                    int64_t n, float* out)
 {
     __shared__ PointTile sm;
@@ -1029,13 +1031,15 @@ void free_cv(wob_cv_s* c)
 cudaError_t launch_quad_D(const CvGeom& g, const float* x, int64_t n, float* out, cudaStream_t s)
 {
     const int threads = 32 * kPointWarps;
-    const int64_t blocks = (n + threads - 1) / threads;  // with a set per warp
-    const int64_t full = grid_for((const void*)k_cv_quad_D<1>, threads, 0, INT64_MAX / 2);
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t full = (int64_t)kPointBlocks * sms;
+    const int64_t blocks = (n + threads - 1) / threads, split = (n + 31) / 32;  // for either form
     if (10 * blocks >= (g.T * (int64_t)g.F <= 256 ? 6 : 19) * full)
-        k_cv_quad_D<1><<<(int)(blocks < full ? blocks : full), threads, 0, s>>>(g, x, n, out);
+        k_cv_quad_D<1><<<(int)std::min(blocks, full), threads, 0, s>>>(g, x, n, out);
     else
-        k_cv_quad_D<kPointWarps><<<grid_for((const void*)k_cv_quad_D<kPointWarps>, threads, 0, n * kPointWarps),
-                                   threads, 0, s>>>(g, x, n, out);
+        k_cv_quad_D<kPointWarps><<<(int)std::min(split, full), threads, 0, s>>>(g, x, n, out);
     return cudaGetLastError();
 }
 
