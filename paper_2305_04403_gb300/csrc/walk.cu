@@ -1020,9 +1020,53 @@ __global__ void k_fwd_mix(WalkParams p, const double* __restrict__ aq_incl, doub
     }
 }
 
+// Start triangle, point and weight a_0 = 2 phi q(z_0) / p(z_0) of a path.
+__device__ __forceinline__ int64_t fwd_start(const WalkParams& p, StreamKey key, uint32_t path,
+                                             int start_mode, const double* wcdf, FFPoint& y, double& a)
+{
+    const double* cdf = start_mode == 1 ? wcdf : p.cdf;
+    const double tot = start_mode == 1 ? wcdf[p.T - 1] : p.area;
+    const u32x4 u = stream_block(key, path, kForwardWalk, 0u, kPurposeArea, 0u, 0u);
+    const long long target = __double_as_longlong(u53(u.x, u.y) * tot);
+    int64_t lo = 0, hi = p.T - 1;
+    while (lo < hi) {
+        const int64_t mid = lo + ((hi - lo) >> 1);
+        if (__double_as_longlong(__ldg(cdf + mid)) > target) hi = mid; else lo = mid + 1;
+    }
+    float b0, b1, b2;
+    frame_point_ff(p, lo, u.z, u.w, y, b0, b1, b2);
+    const double pdf = start_mode == 1
+                           ? ((cdf[lo] - (lo > 0 ? cdf[lo - 1] : 0.0)) / p.tri_n[lo].area) / tot
+                           : 1.0 / p.area;
+    a = 2.0 * (double)p.phi * (double)sl_data_ff(p, lo, y, b0, b1, b2, WOB_BC_NEUMANN, true) / pdf;
+    return lo;
+}
+
+// The starts of every path, for the form with a lane per path: in the engine's
+// hand-out the search and the FP64 quotients run for the few lanes that begin
+// together (1e6 paths of two vertices on 1,280 triangles 698 -> 614 us with this
+// kernel, of eight on 200,000 8.36 -> 7.40 ms; at most 97,000 paths, which begin
+// together anyway, take 3 us more).  The triangle waits in the bits of the path's
+// first coordinate, the weight in its first weight.
+__global__ void __launch_bounds__(128) k_fwd_starts(WalkParams p, int64_t n, int start_mode,
+                                                    const double* __restrict__ wcdf,
+                                                    double* __restrict__ zpos, double* __restrict__ zw)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        FFPoint y;
+        double a;
+        const int64_t j =
+            fwd_start(p, StreamKey{p.key0, p.key1}, (uint32_t)i, start_mode, wcdf, y, a);
+        zpos[3 * i * p.M] = __longlong_as_double((long long)j);
+        zw[i * p.M] = a;
+    }
+}
+
 // The paths as the line engine's walks (p.Q x p.N = paths): a path's weight
 // a_j waits in the first accumulator, its vertices and weights go to zpos
-// and zw.
+// and zw.  STARTED: after k_fwd_starts.
+template <bool STARTED>
 struct FwdPaths : WalkTiles {
     using Base = WalkTiles;
     using Base::p;
@@ -1038,28 +1082,25 @@ struct FwdPaths : WalkTiles {
     template <class Mem>
     __device__ __forceinline__ void begin(const Mem& mem, LaneWalk& lw)
     {
-        const double* cdf = start_mode == 1 ? wcdf : p.cdf;
-        const double tot = start_mode == 1 ? wcdf[p.T - 1] : p.area;
         const uint32_t q = (uint32_t)Base::index(lw);
         mem.set_ids(q, kForwardWalk);
-        const u32x4 u = stream_block(Base::key(lw), q, kForwardWalk, 0u, kPurposeArea, 0u, 0u);
-        const long long target = __double_as_longlong(u53(u.x, u.y) * tot);
-        int64_t lo = 0, hi = p.T - 1;
-        while (lo < hi) {
-            const int64_t mid = lo + ((hi - lo) >> 1);
-            if (__double_as_longlong(__ldg(cdf + mid)) > target) hi = mid; else lo = mid + 1;
-        }
         FFPoint y;
-        float b0, b1, b2;
-        frame_point_ff(p, lo, u.z, u.w, y, b0, b1, b2);
-        const double pdf = start_mode == 1
-                               ? ((cdf[lo] - (lo > 0 ? cdf[lo - 1] : 0.0)) / p.tri_n[lo].area) / tot
-                               : 1.0 / p.area;
-        mem.set(kAccS, 2.0 * (double)p.phi *
-                           (double)sl_data_ff(p, lo, y, b0, b1, b2, WOB_BC_NEUMANN, true) / pdf);
+        int64_t j;
+        if (STARTED) {
+            const int64_t r = Base::index(lw) * p.M;
+            j = __double_as_longlong(zpos[3 * r]);
+            mem.set(kAccS, zw[r]);
+            const u32x4 u = stream_block(Base::key(lw), q, kForwardWalk, 0u, kPurposeArea, 0u, 0u);
+            float b0, b1, b2;
+            frame_point_ff(p, j, u.z, u.w, y, b0, b1, b2);
+        } else {
+            double a;
+            j = fwd_start(p, Base::key(lw), q, start_mode, wcdf, y, a);
+            mem.set(kAccS, a);
+        }
 #pragma unroll
         for (int c = 0; c < 3; ++c) mem.set_x(c, ff_add({y.v0[c], 0.f}, y.p[c]));
-        lw.self = p.inv_order[lo];
+        lw.self = p.inv_order[j];
         lw.k = 0;
         lw.flag = 0;
     }
@@ -1108,15 +1149,15 @@ struct FwdPaths : WalkTiles {
 };
 
 __global__ void __launch_bounds__(kLineThreads, kLineBlocks - 1)
-    k_fwd_lines(WalkParams p, int start_mode, const double* __restrict__ wcdf,
-                double* __restrict__ zpos, double* __restrict__ zw, uint8_t* __restrict__ flags)
+    k_fwd_lines(WalkParams p, double* __restrict__ zpos, double* __restrict__ zw,
+                uint8_t* __restrict__ flags)
 {
     __shared__ LineShared sm;
     extern __shared__ int line_stack[];
     int err = 0;
     WalkCount c{0, 0, 0, 0, 0};
-    FwdPaths pol(p, start_mode, wcdf, zpos, zw, flags);
-    run_lines<FwdPaths, false>(pol, sm.lane(line_stack), sm.vals, p.stack_levels, err, c);
+    FwdPaths<true> pol(p, 0, nullptr, zpos, zw, flags);
+    run_lines<FwdPaths<true>, false>(pol, sm.lane(line_stack), sm.vals, p.stack_levels, err, c);
     if (err) atomicOr(p.error_word, err);
 }
 
@@ -1127,7 +1168,7 @@ __global__ void __launch_bounds__(kGroupThreads, kGroupBlocks)
     __shared__ GroupShared sm;
     extern __shared__ int line_stack[];
     int err = 0;
-    FwdPaths pol(p, start_mode, wcdf, zpos, zw, flags);
+    FwdPaths<false> pol(p, start_mode, wcdf, zpos, zw, flags);
     run_line_groups(pol, sm, line_stack, p.stack_levels, err);
     if (err) atomicOr(p.error_word, err);
 }
@@ -1583,8 +1624,14 @@ int launch_forward(const WalkParams& p, int64_t n_paths, int start_mode, double 
     pp.Q = 1;
     pp.N = (int32_t)n_paths;
     const double* start_cdf = buf ? buf + 3 * p.T : nullptr;
-    int rc = few_walks(pp) ? launch_groups(k_fwd_groups, pp, s, start_mode, start_cdf, zpos, zw, flags)
-                           : launch_lines(k_fwd_lines, pp, s, start_mode, start_cdf, zpos, zw, flags);
+    int rc;
+    if (few_walks(pp)) {
+        rc = launch_groups(k_fwd_groups, pp, s, start_mode, start_cdf, zpos, zw, flags);
+    } else {
+        k_fwd_starts<<<grid_for((const void*)k_fwd_starts, threads, 0, n_paths), threads, 0, s>>>(
+            pp, n_paths, start_mode, start_cdf, zpos, zw);
+        rc = launch_lines(k_fwd_lines, pp, s, zpos, zw, flags);
+    }
     if (buf) cudaFreeAsync(buf, s);
     if (rc == WOB_OK && Q > 0) {
         // packed records and live bytes, then (sum, sum of squares) per split and query
